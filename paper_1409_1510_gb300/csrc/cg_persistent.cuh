@@ -317,9 +317,7 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
                 if (act[0]) raw = __ldcg(reinterpret_cast<const uint4 *>(ax.v.data) + (size_t)s * n + r0);
             site_stencil<PP, 18, R, 1>(g, fat, naik, parity, in, s, 0, r0, act, acc);
             if constexpr (EPI == EPI_PLAIN) {
-#pragma unroll
-                for (int r = 0; r < R; r++)
-                    if (act[r]) store_vec<PP>(vout, s, r0 + r, acc[r]);
+                store_adjacent<PP, R>(vout, s, r0, act, acc);
             } else if constexpr (EPI == EPI_AOP) {
                 Cplx<real> p[R][3];
                 if constexpr (EARLY) {
@@ -331,15 +329,14 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
                 for (int r = 0; r < R; r++) {
                     if (!act[r]) continue;
                     const real m2 = (real)m2v[r0 + r];
-                    Cplx<real> w[3];
+                    Cplx<real>(&w)[3] = acc[r];
                     real d = 0;
 #pragma unroll
                     for (int c = 0; c < 3; c++) {
-                        w[c] = {m2 * p[r][c].re - acc[r][c].re, m2 * p[r][c].im - acc[r][c].im};
+                        w[c] = {m2 * p[r][c].re - w[c].re, m2 * p[r][c].im - w[c].im};
                         d += p[r][c].re * w[c].re + p[r][c].im * w[c].im;
                     }
                     dot[0][r] += (double)d;
-                    store_vec<PP>(vout, s, r0 + r, w);
                     if constexpr (DOTS2) {
                         real f = 0;
 #pragma unroll
@@ -347,6 +344,7 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
                         dot[1][r] += (double)f;
                     }
                 }
+                store_adjacent<PP, R>(vout, s, r0, act, acc);
             } else {
                 static_assert(EPI == EPI_RESID && PP == HISQ_FP64, "residual epilogue is FP64");
                 const VecView<HISQ_FP64> vb{const_cast<void *>(bvec), n};

@@ -349,6 +349,14 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     if (d.n % R != 0) R = 1;
     if (prec == HISQ_FP64 && R > 4) R = 4;  // FP64 kernels are built for up to four RHS per thread
     if (ds && R > 2) R = 2;                 // double-single kernels for up to two
+    // FP32 and BF16 bundles move the R adjacent right-hand sides of a thread as 16-byte words (8 for two
+    // BF16 ones); buffers of the caller's that are aligned to a single element only (8 or 4 bytes) run
+    // one right-hand side per thread
+    const int R_shape = R;
+    if (prec == HISQ_FP32 || prec == HISQ_BF16) {
+        const uintptr_t at = (uintptr_t)d.in | (uintptr_t)d.out | (uintptr_t)d.axpy_in;
+        if (at % (prec == HISQ_BF16 && R == 2 ? 8 : 16) != 0) R = 1;
+    }
     // lane splits exist for 18-real Naik records: two lanes up to four RHS per thread, four up to two
     int S = 1;
     if (!ds && recon == 18 && sh.S == 2 && R <= 4) S = 2;
@@ -420,9 +428,14 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     } else if (d.epi != EPI_PLAIN) {
         size_t need = std::max((size_t)spb * d.n, (size_t)threads + 64);
         smem = need * sizeof(double);
-        // the grid never exceeds one resident wave per SM times 64, nor the tile count
-        if (!d.partials || !d.counter || dslash_partials_needed(a.s1 - a.s0, ctx->num_sms, spb, d.n) > d.partials_cap)
+        // the grid never exceeds one resident wave per SM times 64, nor the tile count (of the launch
+        // shape's R: where alignment halves the sites per block, the scratch bounds the grid instead)
+        int spb_shape = spb, threads_shape;
+        if (R != R_shape) dslash_block_shape(d.n, R_shape, S, sh.threads, true, &spb_shape, &threads_shape);
+        if (!d.partials || !d.counter ||
+            dslash_partials_needed(a.s1 - a.s0, ctx->num_sms, spb_shape, d.n) > d.partials_cap)
             return set_error(HISQ_ERR_ARG, "reduction scratch too small for the Dslash epilogue");
+        a.max_grid = (int)std::min<size_t>(d.partials_cap / d.n, 1u << 30);
     }
     int grid = 0;
     cudaError_t e;

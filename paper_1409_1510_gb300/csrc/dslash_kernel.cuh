@@ -47,6 +47,7 @@ struct KArgs {
     int *err;        // staged kernel: set when a bounded wait for a staged tile runs out
     int s0, s1;      // output sites [s0, s1) of the parity (the whole parity: 0, Vh); the staged
                      // kernel always covers the whole parity
+    int max_grid;    // reducing epilogues: blocks whose partials fit the scratch
 };
 
 template <int P>
@@ -155,19 +156,128 @@ __device__ __forceinline__ void block_reduce_finish(double *red, int rows, int n
     }
 }
 
-// The R neighbour vectors of the active right-hand sides (zeros for the inactive ones).
+// R (2, 4 or 8) consecutive 32-bit words as 8- or 16-byte accesses
+template <int R, bool COHERENT>
+__device__ __forceinline__ void load_words(const uint32_t *p, uint32_t u[R]) {
+    if constexpr (R == 2) {
+        const uint2 x = vld<COHERENT>(reinterpret_cast<const uint2 *>(p));
+        u[0] = x.x;
+        u[1] = x.y;
+    } else {
+#pragma unroll
+        for (int j = 0; j < R / 4; j++) {
+            const uint4 x = vld<COHERENT>(reinterpret_cast<const uint4 *>(p) + j);
+            u[4 * j] = x.x; u[4 * j + 1] = x.y; u[4 * j + 2] = x.z; u[4 * j + 3] = x.w;
+        }
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void store_words(uint32_t *p, const uint32_t u[R]) {
+    if constexpr (R == 2) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(u[0], u[1]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < R / 4; j++)
+            reinterpret_cast<uint4 *>(p)[j] = make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
+    }
+}
+
+// The vectors of the R adjacent right-hand sides r0 .. r0 + R - 1 of one site, R = 2, 4 or 8, in
+// FP32 or BF16: element (s, c, r) is at (s * 3 + c) n + r, so a colour component of all R is one
+// contiguous run of 8 R (FP32) or 4 R (BF16) bytes, read as 8- or 16-byte words (the caller checks
+// the alignment: n and r0 are multiples of R, the base of 16 bytes).  Read one right-hand side at a
+// time, a warp's lanes are 8 R bytes apart and every wavefront of the L1 carries only 1 / R of its
+// bytes: that pipe was 97% busy (FP32, n = 16, R = 2) and bounded every bundle kernel of FP32.
+// Measured one by one / in runs: an FP32 solve of 12 right-hand sides at 48^3 x 12 204 / 172 ms, the FP32
+// Dslash with 13-real Naik links and 4 right-hand sides there 177 / 161 us.
+// All R are read whether active or not: right-hand sides never mix, and those of the inactive ones
+// are not stored.
+template <int P, int R, bool COHERENT>
+__device__ __forceinline__ void load_adjacent(const void *data, int n, long s, int r0, Cplx<float> v[R][3]) {
+    static_assert((P == HISQ_FP32 || P == HISQ_BF16) && R % 2 == 0, "adjacent right-hand sides of plain element layouts");
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const size_t e = ((size_t)s * 3 + c) * n + r0;
+        if constexpr (P == HISQ_FP32) {
+            const float4 *d = reinterpret_cast<const float4 *>(reinterpret_cast<const float2 *>(data) + e);
+#pragma unroll
+            for (int j = 0; j < R / 2; j++) {
+                const float4 x = vld<COHERENT>(d + j);
+                v[2 * j][c] = {x.x, x.y};
+                v[2 * j + 1][c] = {x.z, x.w};
+            }
+        } else {
+            const uint32_t *d = reinterpret_cast<const uint32_t *>(data) + e;
+            uint32_t u[R];
+            load_words<R, COHERENT>(d, u);
+#pragma unroll
+            for (int r = 0; r < R; r++)  // a bf16 is the top half of its float
+                v[r][c] = {__uint_as_float(u[r] << 16), __uint_as_float(u[r] & 0xffff0000u)};
+        }
+    }
+}
+
+// whether R adjacent right-hand sides of precision P are moved as one run per colour component
+template <int P, int R>
+__host__ __device__ constexpr bool adjacent_io() {
+    return (P == HISQ_FP32 || P == HISQ_BF16) && R % 2 == 0;
+}
+
+// The R neighbour vectors of the active right-hand sides (zeros for the inactive ones where they
+// are read one by one).
 template <int P, int R, bool COHERENT>
 __device__ __forceinline__ void load_neighbours(const VecView<P> &vin, int nb, int r0, const bool act[R],
                                                 Cplx<typename Prec<P>::real> v[R][3]) {
+    if constexpr (adjacent_io<P, R>()) {
+        load_adjacent<P, R, COHERENT>(vin.data, vin.n, nb, r0, v);
+    } else {
 #pragma unroll
-    for (int r = 0; r < R; r++) {
-        if (act[r]) {
-            load_vec<P, COHERENT>(vin, nb, r0 + r, v[r]);
-        } else {
+        for (int r = 0; r < R; r++) {
+            if (act[r]) {
+                load_vec<P, COHERENT>(vin, nb, r0 + r, v[r]);
+            } else {
 #pragma unroll
-            for (int c = 0; c < 3; c++) v[r][c] = {0, 0};
+                for (int c = 0; c < 3; c++) v[r][c] = {0, 0};
+            }
         }
     }
+}
+
+// stores the R vectors of the right-hand sides r0 .. of one site where act[r]; runs of adjacent
+// right-hand sides as in load_adjacent when all are active
+template <int P, int R>
+__device__ __forceinline__ void store_adjacent(const VecView<P> &v, long s, int r0, const bool act[R],
+                                               const Cplx<typename Prec<P>::real> w[R][3]) {
+    if constexpr (adjacent_io<P, R>()) {
+        bool all = true;
+#pragma unroll
+        for (int r = 0; r < R; r++) all = all && act[r];
+        if (all) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const size_t e = ((size_t)s * 3 + c) * v.n + r0;
+                if constexpr (P == HISQ_FP32) {
+                    float4 *d = reinterpret_cast<float4 *>(reinterpret_cast<float2 *>(v.data) + e);
+#pragma unroll
+                    for (int j = 0; j < R / 2; j++)
+                        d[j] = make_float4(w[2 * j][c].re, w[2 * j][c].im, w[2 * j + 1][c].re, w[2 * j + 1][c].im);
+                } else {
+                    uint32_t u[R];
+#pragma unroll
+                    for (int r = 0; r < R; r++) {
+                        const __nv_bfloat162 b = __floats2bfloat162_rn(w[r][c].re, w[r][c].im);
+                        u[r] = *reinterpret_cast<const uint32_t *>(&b);
+                    }
+                    store_words<R>(reinterpret_cast<uint32_t *>(v.data) + e, u);
+                }
+            }
+            return;
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; r++)
+        if (act[r]) store_vec<P>(v, s, r0 + r, w[r]);
 }
 
 // Input of the stencil: the colour vectors of one bundle as stored (COHERENT: read through L2,
@@ -243,19 +353,20 @@ __device__ __forceinline__ void load_pairs(const void *data, int n, int nb, int 
         }
     } else {
         static_assert(P == HISQ_BF16, "paired loads for 16-bit storage");
-        // element (s, c, r) is the bf16 pair (re, im) at (s * 3 + c) n + r: two adjacent right-hand
-        // sides are one 8-byte word; a bf16 is the top half of its float
+        // element (s, c, r) is the bf16 pair (re, im) at (s * 3 + c) n + r: the 2 Q2 adjacent right-hand
+        // sides are one run of words; a bf16 is the top half of its float
         const uint32_t *e = reinterpret_cast<const uint32_t *>(data);
 #pragma unroll
-        for (int q = 0; q < Q2; q++)
+        for (int c = 0; c < 3; c++) {
+            uint32_t u[2 * Q2];
+            load_words<2 * Q2, COHERENT>(e + ((size_t)nb * 3 + c) * n + r0, u);
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const size_t idx = ((size_t)nb * 3 + c) * n + r0 + 2 * q;
-                const uint32_t a = act[2 * q] ? vld<COHERENT>(e + idx) : 0u;
-                const uint32_t b = act[2 * q + 1] ? vld<COHERENT>(e + idx + 1) : 0u;
+            for (int q = 0; q < Q2; q++) {
+                const uint32_t a = u[2 * q], b = u[2 * q + 1];
                 vr[q][c] = f2(__uint_as_float(a << 16), __uint_as_float(b << 16));
                 vi[q][c] = f2(__uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u));
             }
+        }
     }
 }
 
@@ -496,26 +607,24 @@ __global__ void __launch_bounds__(256) dslash_kernel(KArgs a) {
 
         // ---- epilogue ----
         if constexpr (EPI == EPI_PLAIN) {
-#pragma unroll
-            for (int r = 0; r < R; r++)
-                if (act[r]) store_vec<P>(vout, s, r0 + r, acc[r]);
+            store_adjacent<P, R>(vout, s, r0, act, acc);
         } else if constexpr (EPI == EPI_AOP) {
             const VecView<P> vp = view<P>(a.axpy, g.Vh, a.n);
             const real m2 = (real)a.mass2;
+            Cplx<real> p[R][3];
+            load_neighbours<P, R, false>(vp, s, r0, act, p);
 #pragma unroll
             for (int r = 0; r < R; r++) {
                 if (!act[r]) continue;
-                Cplx<real> p[3], w[3];
-                load_vec<P>(vp, s, r0 + r, p);
                 real d = 0;
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    w[c] = {m2 * p[c].re - acc[r][c].re, m2 * p[c].im - acc[r][c].im};
-                    d += p[c].re * w[c].re + p[c].im * w[c].im;
+                    acc[r][c] = {m2 * p[r][c].re - acc[r][c].re, m2 * p[r][c].im - acc[r][c].im};
+                    d += p[r][c].re * acc[r][c].re + p[r][c].im * acc[r][c].im;
                 }
                 dot[r] += (double)d;
-                store_vec<P>(vout, s, r0 + r, w);
             }
+            store_adjacent<P, R>(vout, s, r0, act, acc);
         } else {
             static_assert(EPI == EPI_RESID && P == HISQ_FP64, "residual epilogue is FP64 only");
             const VecView<HISQ_FP64> vx = view<HISQ_FP64>(a.axpy, g.Vh, a.n);
@@ -711,9 +820,7 @@ __global__ void __launch_bounds__(512, 1) dslash_staged_kernel(KArgs a) {
                 }
         if (valid && part == 0) {
             if constexpr (EPI == EPI_PLAIN) {
-#pragma unroll
-                for (int r = 0; r < R; r++)
-                    if (act[r]) store_vec<P>(vout, s, r0 + r, acc[r]);
+                store_adjacent<P, R>(vout, s, r0, act, acc);
             } else {
                 static_assert(EPI == EPI_AOP, "the staged kernel has the plain and A-operator epilogues");
                 const VecView<P> vp = view<P>(a.axpy, g.Vh, a.n);

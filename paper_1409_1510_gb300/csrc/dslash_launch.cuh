@@ -28,6 +28,7 @@ inline cudaError_t launch_one(const KArgs &a, int threads, size_t smem, int num_
     int grid = wave_grid(k, threads, smem, num_sms, tiles);
     // one full wave, every block with the same number of tiles
     grid = (int)balanced_grid(tiles, grid);
+    if (EPI != EPI_PLAIN) grid = std::min(grid, a.max_grid);
     if (grid_out) *grid_out = grid;
     k<<<grid, threads, smem, stream>>>(a);
     return cudaGetLastError();

@@ -203,3 +203,27 @@ def test_fma_peaks_are_measured():
     with gpu((4, 4, 4, 4), 1, 18) as g:
         f32, f64 = g.hisq.hisq_measure_fma_peaks()
         assert 1.0 < f32 < 1000.0 and 0.01 < f64 < 1000.0 and f32 > 4 * f64
+
+
+@pytest.mark.parametrize("prec,n", [(1, 2), (1, 4), (1, 64), (3, 2), (3, 4), (3, 12), (3, 16)])
+def test_element_aligned_buffers(prec, n):
+    """Bundles at an address aligned to one element only (8 bytes FP32, 4 BF16) give what aligned ones do:
+    the wide loads of adjacent right-hand sides are taken only where the addresses allow them."""
+    dims, mass, step = (6, 4, 8, 4), 0.2, {1: 8, 3: 4}[prec]
+    with gpu(dims, prec, 18) as g:
+        v = _rhs(g.lat, n, 300)
+        vin, w, a = g.pack(v), g.bundle(n), g.bundle(n)
+        size = vin.numel()
+        off = [g.torch.empty(size + 16, dtype=g.torch.uint8, device=g.dev)[step:step + size] for _ in range(2)]
+        off[0].copy_(vin)
+        assert off[0].data_ptr() % 16 == step
+        pap, pap_off = np.zeros(n), np.zeros(n)
+        for call in (g.hisq.hisq_aop, g.hisq.hisq_aop_noalloc):
+            call(g.fat, g.naik, mass, vin, a, n, pap)
+            call(g.fat, g.naik, mass, off[0], off[1], n, pap_off)
+            # the same sums in the same order per right-hand side; the dots only regroup FP64 partials
+            assert rel_err(g.unpack(off[1].clone(), n), g.unpack(a, n)) <= {1: 1e-6, 3: 4e-3}[prec]
+            assert np.allclose(pap_off, pap, rtol=1e-5)
+        g.hisq.hisq_dslash(g.fat, g.naik, vin, w, n, 1)
+        g.hisq.hisq_dslash(g.fat, g.naik, off[0], off[1], n, 1)
+        assert rel_err(g.unpack(off[1].clone(), n), g.unpack(w, n)) <= {1: 1e-6, 3: 4e-3}[prec]
