@@ -122,11 +122,15 @@ __device__ __forceinline__ void block_reduce_finish(double *red, int rows, int n
             if (tid < ndots) red[tid] = red[blockDim.x + tid];
         } else {
             // many columns (network weight gradients): one thread per column
+            // (four sums in flight: an FP64 add is a 64-cycle dependent operation)
             for (int j = tid; j < ndots; j += blockDim.x) {
-                double t = 0.0;
-#pragma unroll 8
-                for (int b = 0; b < nb; b++) t += __ldcg(ra.partials + (size_t)b * ndots + j);
-                red[ndots + j] = t;
+                double t[4] = {0.0, 0.0, 0.0, 0.0};
+                int b = 0;
+                for (; b + 4 <= nb; b += 4)
+#pragma unroll
+                    for (int u = 0; u < 4; u++) t[u] += __ldcg(ra.partials + (size_t)(b + u) * ndots + j);
+                for (; b < nb; b++) t[0] += __ldcg(ra.partials + (size_t)b * ndots + j);
+                red[ndots + j] = (t[0] + t[1]) + (t[2] + t[3]);
             }
             __syncthreads();
             for (int j = tid; j < ndots; j += blockDim.x) red[j] = red[ndots + j];

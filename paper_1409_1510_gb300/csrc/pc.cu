@@ -211,14 +211,17 @@ static int run_layer(hisq_ctx *ctx, const hisq_links *naik, const PcLayerArgs &p
 }
 
 template <int A, int B>
-static int run_grad(hisq_ctx *ctx, const hisq_links *naik, PcWork &w, const PcGradArgs &ga, cudaStream_t st) {
+static int run_grad(hisq_ctx *ctx, const hisq_links *naik, PcWork &w, PcGradArgs ga, cudaStream_t st) {
     constexpr int ND = PC_PATHS * A * B * 2;
-    size_t smem = (size_t)8 * ND * sizeof(double);
+    const size_t smem = std::max(2 * ND, 32 * PC_GRAD_WARPS + 64) * sizeof(double);
+    // a tile gives every lane eight (site, sample) pairs per path, fewer where the lattice would not
+    // fill the GPU
+    const int rows = 32 / ga.L.K;
+    ga.L.spb = rows * (int)std::max(1L, std::min(8L, (long)ctx->geom.Vh / ((long)rows * ctx->num_sms * 2)));
     auto launch = [&](auto k) -> int {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int grid = grid_of(ctx, k, smem, ga.L.spb);
         if ((size_t)grid * ND > w.partials_cap) grid = (int)(w.partials_cap / ND);
-        k<<<grid, 256, smem, st>>>(ga);
+        k<<<grid, 32 * PC_GRAD_WARPS, smem, st>>>(ga);
         return HISQ_OK;
     };
     switch (naik->recon) {

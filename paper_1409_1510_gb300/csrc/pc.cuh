@@ -39,10 +39,11 @@ struct PcLayerArgs {
 };
 
 // Weights in shared memory as ws[q][b][a] for q = 0 (identity) and q = 1 + slot (16 slots),
-// with the backward-slot sign folded in.  ADJ: the adjoint of a layer with weights W[17][A][B]
-// (mapping B -> A channels): ws[q][b][a] = conj(W[adj(q)][a][b]).
+// with the backward-slot sign folded in, each complex weight as (re, re, im, im): the two packed
+// operands of mix().  ADJ: the adjoint of a layer with weights W[17][A][B] (mapping B -> A
+// channels): ws[q][b][a] = conj(W[adj(q)][a][b]).
 template <int A, int B, bool ADJ>
-__device__ __forceinline__ void stage_weights(const float2 *W, float2 *ws) {
+__device__ __forceinline__ void stage_weights(const float2 *W, float4 *ws) {
     for (int i = threadIdx.x; i < PC_PATHS * A * B; i += blockDim.x) {
         int q = i / (A * B), rem = i - q * A * B, b = rem / A, a = rem - b * A;
         int path = q == 0 ? 0 : slot_path(q - 1);
@@ -54,65 +55,83 @@ __device__ __forceinline__ void stage_weights(const float2 *W, float2 *ws) {
         } else {
             w = W[(path * B + b) * A + a];
         }
-        ws[i] = make_float2(sign * w.x, sign * w.y);
+        ws[i] = make_float4(sign * w.x, sign * w.x, sign * w.y, sign * w.y);
     }
 }
 
+// Channels of a field with C channels that are worked on together: two of four (one 16-byte load
+// per colour), or the only one.  Loaded channel by channel, a warp's lanes are 32 bytes apart and every
+// wavefront of the L1 carries a quarter of its bytes: that pipe was 73% (4 -> 4) and 93% (4 -> 1) busy.
+// M^dag M on 16 vectors at 32^3 x 8, FP32 arithmetic bound from then on: 4.57 / 3.52 ms.
 template <int C>
-__device__ __forceinline__ void load_channels(const float2 *f, int s, int k, int K, Cplx<float> h[C][3]) {
+constexpr int PC_CHUNK = C == 4 ? 2 : 1;
+
+// channels a0 .. a0 + PC_CHUNK<C> - 1 of sample k at site s (four-channel fields are the library's
+// own, 16-byte aligned)
+template <int C>
+__device__ __forceinline__ void load_chunk(const float2 *f, int s, int k, int K, int a0, float2 h[PC_CHUNK<C>][3]) {
 #pragma unroll
-    for (int c = 0; c < 3; c++)
-#pragma unroll
-        for (int a = 0; a < C; a++) {
-            float2 v = __ldg(f + (((size_t)s * 3 + c) * K + k) * C + a);
-            h[a][c] = {v.x, v.y};
+    for (int c = 0; c < 3; c++) {
+        const size_t e = (((size_t)s * 3 + c) * K + k) * C + a0;
+        if constexpr (C == 4) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(f + e));
+            h[0][c] = make_float2(v.x, v.y);
+            h[1][c] = make_float2(v.z, v.w);
+        } else {
+            static_assert(C == 1, "fields have one or four channels");
+            h[0][c] = __ldg(f + e);
         }
+    }
 }
 
-// y = M h for every channel
-template <int C>
-__device__ __forceinline__ void transport(const Cplx<float> M[3][3], const Cplx<float> h[C][3], Cplx<float> y[C][3]) {
+// y = M h for N channels
+template <int N>
+__device__ __forceinline__ void transport(const Cplx<float> M[3][3], const float2 h[N][3], float2 y[N][3]) {
 #pragma unroll
-    for (int a = 0; a < C; a++)
+    for (int a = 0; a < N; a++)
 #pragma unroll
         for (int r = 0; r < 3; r++) {
             float re = 0.f, im = 0.f;
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                re = fmaf(M[r][c].re, h[a][c].re, fmaf(-M[r][c].im, h[a][c].im, re));
-                im = fmaf(M[r][c].re, h[a][c].im, fmaf(M[r][c].im, h[a][c].re, im));
+                re = fmaf(M[r][c].re, h[a][c].x, fmaf(-M[r][c].im, h[a][c].y, re));
+                im = fmaf(M[r][c].re, h[a][c].y, fmaf(M[r][c].im, h[a][c].x, im));
             }
-            y[a][r] = {re, im};
+            y[a][r] = make_float2(re, im);
         }
 }
 
-template <int A, int B>
-__device__ __forceinline__ void mix(const float2 *ws, const Cplx<float> y[A][3], Cplx<float> acc[B][3]) {
+// The output sum of a layer as packed pairs: with w = (wr, wi) and y = (yr, yi),
+// P += (wr, wr) y and N += (wi, wi) y are two packed FMAs per complex product in place of four
+// scalar ones, and the output is (P.x - N.y, P.y + N.x).
+template <int B>
+struct MixAcc {
+    float2 P[B][3], N[B][3];
+};
+
+// channels a0 .. a0 + N - 1 of the A input channels, all B output channels
+template <int A, int B, int N>
+__device__ __forceinline__ void mix(const float4 *ws, int a0, const float2 y[N][3], MixAcc<B> &acc) {
 #pragma unroll
-    for (int b = 0; b < B; b++)
+    for (int a = 0; a < N; a++)
 #pragma unroll
-        for (int a = 0; a < A; a++) {
-            float2 w = ws[b * A + a];
+        for (int b = 0; b < B; b++) {
+            const float4 w = ws[b * A + a0 + a];
+            const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.z, w.w);
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                acc[b][c].re = fmaf(w.x, y[a][c].re, fmaf(-w.y, y[a][c].im, acc[b][c].re));
-                acc[b][c].im = fmaf(w.x, y[a][c].im, fmaf(w.y, y[a][c].re, acc[b][c].im));
+                acc.P[b][c] = __ffma2_rn(wr, y[a][c], acc.P[b][c]);
+                acc.N[b][c] = __ffma2_rn(wi, y[a][c], acc.N[b][c]);
             }
         }
 }
 
-// Calls f(q, u) for q = 0 (u = h at the site) and q = 1 + slot (u = L_slot h(neighbour)).
-template <int A, int NR, typename F>
-__device__ __forceinline__ void for_each_path(const PcLayerArgs &p, int s, int k, F &&f) {
+// Calls f(q, M, nb) for every link of the site: q = 1 + slot, M the gathered link, nb the neighbour.
+template <int NR, typename F>
+__device__ __forceinline__ void for_each_link(const PcLayerArgs &p, int s, F &&f) {
     using FatC = LinkCodec<HISQ_FP32, 18>;
     using NaikC = LinkCodec<HISQ_FP32, NR>;
     const Geom &g = p.g;
-    if (p.in_same) {
-        Cplx<float> h[A][3];
-        load_channels<A>(p.in_same, s, k, p.K, h);
-        f(0, h);
-    }
-    if (!p.in_opp) return;
     const SiteCoord sc = decode_site(g, s, p.parity);
 #pragma unroll
     for (int grp = 0; grp < FatC::GROUPS; grp++) {
@@ -124,10 +143,7 @@ __device__ __forceinline__ void for_each_path(const PcLayerArgs &p, int s, int k
             const int nb = neighbour(g, sc, s, slot >> 1, (slot & 1) ? -1 : 1);
             Cplx<float> M[3][3];
             FatC::decode(u, l, M);
-            Cplx<float> h[A][3], y[A][3];
-            load_channels<A>(p.in_opp, nb, k, p.K, h);
-            transport<A>(M, h, y);
-            f(1 + slot, y);
+            f(1 + slot, M, nb);
         }
     }
 #pragma unroll
@@ -140,116 +156,229 @@ __device__ __forceinline__ void for_each_path(const PcLayerArgs &p, int s, int k
             const int nb = neighbour(g, sc, s, slot >> 1, (slot & 1) ? -3 : 3);
             Cplx<float> M[3][3];
             NaikC::decode(u, l, M);
-            Cplx<float> h[A][3], y[A][3];
-            load_channels<A>(p.in_opp, nb, k, p.K, h);
-            transport<A>(M, h, y);
-            f(9 + slot, y);
+            f(9 + slot, M, nb);
         }
     }
 }
 
+// Resident blocks per SM that the register budget is set for: 24 warps for the four-to-one layer of
+// 18-real links, 16 for the others (more would spill).
+constexpr int pc_layer_blocks(int A, int B, int NR) { return A == 4 && B == 1 && NR == 18 ? 3 : 2; }
+
 // one thread per (site, sample); K threads share a site's links
 template <int A, int B, bool ADJ, int NR>
-__global__ void __launch_bounds__(256) pc_layer_kernel(PcLayerArgs p) {
-    __shared__ float2 ws[PC_PATHS * A * B];
+__global__ void __launch_bounds__(256, pc_layer_blocks(A, B, NR)) pc_layer_kernel(PcLayerArgs p) {
+    constexpr int N = PC_CHUNK<A>;
+    __shared__ float4 ws[PC_PATHS * A * B];
     stage_weights<A, B, ADJ>(p.W, ws);
     __syncthreads();
     const int k = threadIdx.x % p.K, sl = threadIdx.x / p.K;
     for (int tile = blockIdx.x; (long)tile * p.spb < p.g.Vh; tile += gridDim.x) {
         const int s = tile * p.spb + sl;
         if (s >= p.g.Vh || sl >= p.spb) continue;
-        Cplx<float> acc[B][3];
+        MixAcc<B> acc;
 #pragma unroll
         for (int b = 0; b < B; b++)
 #pragma unroll
-            for (int c = 0; c < 3; c++) acc[b][c] = {0.f, 0.f};
-        for_each_path<A, NR>(p, s, k, [&](int q, const Cplx<float>(&y)[A][3]) { mix<A, B>(ws + q * A * B, y, acc); });
+            for (int c = 0; c < 3; c++) acc.P[b][c] = acc.N[b][c] = make_float2(0.f, 0.f);
+        if (p.in_same) {
 #pragma unroll
-        for (int c = 0; c < 3; c++)
+            for (int a0 = 0; a0 < A; a0 += N) {
+                float2 h[N][3];
+                load_chunk<A>(p.in_same, s, k, p.K, a0, h);
+                mix<A, B, N>(ws, a0, h, acc);
+            }
+        }
+        if (p.in_opp) {
+            for_each_link<NR>(p, s, [&](int q, const Cplx<float>(&M)[3][3], int nb) {
 #pragma unroll
-            for (int b = 0; b < B; b++) p.out[(((size_t)s * 3 + c) * p.K + k) * B + b] = make_float2(acc[b][c].re, acc[b][c].im);
+                for (int a0 = 0; a0 < A; a0 += N) {
+                    float2 h[N][3], y[N][3];
+                    load_chunk<A>(p.in_opp, nb, k, p.K, a0, h);
+                    transport<N>(M, h, y);
+                    mix<A, B, N>(ws + q * A * B, a0, y, acc);
+                }
+            });
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            float2 o[B];
+#pragma unroll
+            for (int b = 0; b < B; b++)
+                o[b] = make_float2(acc.P[b][c].x - acc.N[b][c].y, acc.P[b][c].y + acc.N[b][c].x);
+            const size_t e = (((size_t)s * 3 + c) * p.K + k) * B;
+            if constexpr (B == 4) {
+                float4 *d = reinterpret_cast<float4 *>(p.out + e);
+                d[0] = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
+                d[1] = make_float4(o[2].x, o[2].y, o[3].x, o[3].y);
+            } else {
+                p.out[e] = o[0];
+            }
+        }
     }
 }
 
 // Weight gradient of a layer A -> B channels at one output parity:
 //   gW[path][b][a] += sum_x sum_colour G_b(x) conj((T_path h_a)(x))   (summed over samples)
 // G: [Vh][3][K][B] at the output parity.  Result: 17*B*A complex numbers (doubles) in dot_out,
-// in the weight layout [path][b][a].  Deterministic: warp shuffles, fixed-order block and grid
-// sums (last-block-done), FP64 above the warp.
+// in the weight layout [path][b][a].
+//
+// Each of the block's eight warps owns one direction of one link kind (its two hops are two
+// paths), and the warps take turns at the identity path, so a path's 2 A B sums stay in the
+// registers of one warp: over a tile of p.spb sites every lane sums its (site, sample) pairs in
+// FP32, then one transposing shuffle tree (2 A B - 1 shuffles) leaves component i of the warp's sum
+// in lane i, which adds it to its FP64 sum.  A lane-by-lane reduction of every component of every
+// site, with lane 0 adding into FP64 sums in shared memory, was bound by those additions (75% of
+// the FP64 pipe, 5 ms for a 4 -> 4 layer): at 32^3 x 8 with 16 samples the loss and gradient took
+// 37.6 ms, with this kernel and the packed layers above 17.8 ms.
 struct PcGradArgs {
-    PcLayerArgs L;       // in_same, in_opp: the layer input h; out unused
+    PcLayerArgs L;       // in_same, in_opp: the layer input h; spb: sites per tile; out unused
     const float2 *G;     // gradient w.r.t. the layer output at the output parity
     RedArgs red;
 };
 
-template <int A, int B, int NR>
-__global__ void __launch_bounds__(256) pc_grad_kernel(PcGradArgs ga) {
-    constexpr int ND = PC_PATHS * A * B * 2;  // doubles per partial
-    extern __shared__ double red[];
-    const PcLayerArgs &p = ga.L;
-    const int k = threadIdx.x % p.K, sl = threadIdx.x / p.K;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nwarps = blockDim.x >> 5;
-    // per-thread accumulators for all paths would not fit in registers: accumulate each path's
-    // products across the thread's sites first (loop over sites inside the path loop is not
-    // possible since paths are produced per site), so reduce per site visit into shared memory.
-    for (int i = threadIdx.x; i < nwarps * ND; i += blockDim.x) red[i] = 0.0;
-    __syncthreads();
-    for (int tile = blockIdx.x; (long)tile * p.spb < p.g.Vh; tile += gridDim.x) {
-        const int s = tile * p.spb + sl;
-        const bool valid = s < p.g.Vh && sl < p.spb;
-        Cplx<float> G[B][3];
-        if (valid) {
-            load_channels<B>(ga.G, s, k, p.K, G);
-        } else {
+constexpr int PC_GRAD_WARPS = 8;  // four directions of two link kinds
+
+// v[0 .. N): in lane l afterwards v[0] = the warp's sum of component l % N (N a power of two <= 32)
+template <int N>
+__device__ __forceinline__ void transpose_sum(float v[N], int lane) {
 #pragma unroll
-            for (int b = 0; b < B; b++)
+    for (int n = N; n > 1; n /= 2) {
+        const int off = n / 2;
+        const bool up = (lane & off) != 0;
 #pragma unroll
-                for (int c = 0; c < 3; c++) G[b][c] = {0.f, 0.f};
-        }
-        auto body = [&](int q, const Cplx<float>(&y)[A][3]) {
-            const int path = q == 0 ? 0 : slot_path(q - 1);
-            const float sign = q == 0 ? 1.0f : slot_sign(q - 1);
-#pragma unroll
-            for (int b = 0; b < B; b++)
-#pragma unroll
-                for (int a = 0; a < A; a++) {
-                    float re = 0.f, im = 0.f;
-#pragma unroll
-                    for (int c = 0; c < 3; c++) {  // G conj(y)
-                        re += G[b][c].re * y[a][c].re + G[b][c].im * y[a][c].im;
-                        im += G[b][c].im * y[a][c].re - G[b][c].re * y[a][c].im;
-                    }
-                    re *= sign;
-                    im *= sign;
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) {
-                        re += __shfl_xor_sync(0xffffffffu, re, off);
-                        im += __shfl_xor_sync(0xffffffffu, im, off);
-                    }
-                    if (lane == 0) {
-                        double *d = red + warp * ND + ((path * B + b) * A + a) * 2;
-                        d[0] += (double)re;
-                        d[1] += (double)im;
-                    }
-                }
-        };
-        // every lane of a warp must reach the shuffles: invalid lanes contribute zeros
-        if (valid) {
-            for_each_path<A, NR>(p, s, k, body);
-        } else {
-            // mirror the path sequence of valid lanes with zero products
-            Cplx<float> z[A][3];
-#pragma unroll
-            for (int a = 0; a < A; a++)
-#pragma unroll
-                for (int c = 0; c < 3; c++) z[a][c] = {0.f, 0.f};
-            if (p.in_same) body(0, z);
-            if (p.in_opp)
-                for (int q = 1; q <= 16; q++) body(q, z);
+        for (int i = 0; i < n / 2; i++) {
+            const float keep = up ? v[i + off] : v[i], send = up ? v[i] : v[i + off];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
         }
     }
-    block_reduce_finish(red, nwarps, ND, 0, ga.red);
+#pragma unroll
+    for (int off = N; off < 32; off *= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+}
+
+// acc[(b A + a) 2 ..] += sum_colour G_b conj(y_a) for channels a0 .. a0 + N - 1
+template <int A, int B, int N>
+__device__ __forceinline__ void outer_acc(const float2 G[B][3], const float2 y[N][3], int a0, float *acc) {
+#pragma unroll
+    for (int a = 0; a < N; a++)
+#pragma unroll
+        for (int b = 0; b < B; b++) {
+            float &re = acc[(b * A + a0 + a) * 2], &im = acc[(b * A + a0 + a) * 2 + 1];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                re = fmaf(G[b][c].x, y[a][c].x, fmaf(G[b][c].y, y[a][c].y, re));
+                im = fmaf(G[b][c].y, y[a][c].x, fmaf(-G[b][c].x, y[a][c].y, im));
+            }
+        }
+}
+
+template <int C>
+__device__ __forceinline__ void load_all(const float2 *f, int s, int k, int K, float2 h[C][3]) {
+#pragma unroll
+    for (int a0 = 0; a0 < C; a0 += PC_CHUNK<C>) load_chunk<C>(f, s, k, K, a0, h + a0);
+}
+
+// link 2 mu + DIR of a record (mu known at run time, the same for the whole warp)
+template <int NR, int DIR>
+__device__ __forceinline__ void load_direction(const LinkField &f, int parity, int Vh, int s, int mu,
+                                               Cplx<float> M[3][3]) {
+    using C = LinkCodec<HISQ_FP32, NR>;
+    uint32_t u[C::WG * 4];
+    C::load_group(f, parity, Vh, s, 2 * mu / C::G, u);
+    if constexpr (C::G == 2) {
+        C::decode(u, DIR, M);
+    } else {
+        static_assert(C::G == 4, "records of two or four links per group");
+        if (mu & 1) C::decode(u, 2 + DIR, M);
+        else C::decode(u, DIR, M);
+    }
+}
+
+template <int A, int B, int NR, int DIR>
+__device__ __forceinline__ double grad_hop(const PcGradArgs &ga, const LinkField &f, int hop, int mu, int s0, int s1,
+                                           int row, int rows, int k, int lane) {
+    constexpr int N = PC_CHUNK<A>, NV = 2 * A * B;
+    const PcLayerArgs &p = ga.L;
+    float acc[NV];
+#pragma unroll
+    for (int i = 0; i < NV; i++) acc[i] = 0.f;
+    if (row < rows) {
+        for (int s = s0 + row; s < s1; s += rows) {
+            Cplx<float> M[3][3];
+            load_direction<NR, DIR>(f, p.parity, p.g.Vh, s, mu, M);
+            const SiteCoord sc = decode_site(p.g, s, p.parity);
+            const int nb = neighbour_rt(p.g, sc, s, mu, DIR ? -hop : hop);
+            float2 G[B][3];
+            load_all<B>(ga.G, s, k, p.K, G);
+#pragma unroll
+            for (int a0 = 0; a0 < A; a0 += N) {
+                float2 h[N][3], y[N][3];
+                load_chunk<A>(p.in_opp, nb, k, p.K, a0, h);
+                transport<N>(M, h, y);
+                outer_acc<A, B, N>(G, y, a0, acc);
+            }
+        }
+    }
+    transpose_sum<NV>(acc, lane);
+    return (double)acc[0];
+}
+
+template <int A, int B, int NR>
+__global__ void __launch_bounds__(32 * PC_GRAD_WARPS, 2) pc_grad_kernel(PcGradArgs ga) {
+    constexpr int N = PC_CHUNK<A>, NV = 2 * A * B, ND = PC_PATHS * NV;  // doubles per partial
+    extern __shared__ double red[];
+    __shared__ double same[PC_GRAD_WARPS][NV];
+    const PcLayerArgs &p = ga.L;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = 32 / p.K, k = lane % p.K, row = lane / p.K;  // (site, sample) pairs of a warp
+    const int mu = warp & 3;
+    const bool naik_kind = warp >= 4;
+    double fwd = 0.0, bwd = 0.0, idn = 0.0;
+    int turn = 0;
+    for (int tile = blockIdx.x; (long)tile * p.spb < p.g.Vh; tile += gridDim.x, turn++) {
+        const int s0 = tile * p.spb, s1 = min(s0 + p.spb, p.g.Vh);
+        if (p.in_opp) {
+            if (naik_kind) {
+                fwd += grad_hop<A, B, NR, 0>(ga, p.naik, 3, mu, s0, s1, row, rows, k, lane);
+                bwd += grad_hop<A, B, NR, 1>(ga, p.naik, 3, mu, s0, s1, row, rows, k, lane);
+            } else {
+                fwd += grad_hop<A, B, 18, 0>(ga, p.fat, 1, mu, s0, s1, row, rows, k, lane);
+                bwd += grad_hop<A, B, 18, 1>(ga, p.fat, 1, mu, s0, s1, row, rows, k, lane);
+            }
+        }
+        if (p.in_same && (turn & (PC_GRAD_WARPS - 1)) == warp) {
+            float acc[NV];
+#pragma unroll
+            for (int i = 0; i < NV; i++) acc[i] = 0.f;
+            if (row < rows) {
+                for (int s = s0 + row; s < s1; s += rows) {
+                    float2 G[B][3];
+                    load_all<B>(ga.G, s, k, p.K, G);
+#pragma unroll
+                    for (int a0 = 0; a0 < A; a0 += N) {
+                        float2 h[N][3];
+                        load_chunk<A>(p.in_same, s, k, p.K, a0, h);
+                        outer_acc<A, B, N>(G, h, a0, acc);
+                    }
+                }
+            }
+            transpose_sum<NV>(acc, lane);
+            idn += (double)acc[0];
+        }
+    }
+    if (lane < NV) {
+        const int path = slot_path(2 * mu + (naik_kind ? 8 : 0));  // forward hop; the backward one follows
+        red[path * NV + lane] = fwd;
+        red[(path + 1) * NV + lane] = -bwd;                        // backward slots hold -U^dag
+        same[warp][lane] = idn;
+    }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double s = 0.0;
+        for (int w = 0; w < PC_GRAD_WARPS; w++) s += same[w][threadIdx.x];
+        red[threadIdx.x] = s;
+    }
+    block_reduce_finish(red, 1, ND, 0, ga.red);
 }
 
 }  // namespace hisq
