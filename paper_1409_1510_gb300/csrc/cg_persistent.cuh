@@ -117,8 +117,10 @@ __device__ __forceinline__ bool grid_sync(const PersArgs &a) {
 }
 
 // Largest block: 1024 threads at one right-hand side per thread (64 registers), 512 otherwise
-// (128 registers); the launch may use fewer (a multiple of 32 dividing into the SM's resources).
-__host__ __device__ constexpr int pers_threads(int R) { return R == 1 ? 1024 : 512; }
+// or with four lanes per site (128 registers); the launch may use fewer (a multiple of 32 dividing into
+// the SM's resources).
+__host__ __device__ constexpr int pers_threads(int R, int S = 1) { return R == 1 && S == 1 ? 1024 : 512; }
+constexpr int PERS_SPLIT = -4;  // "R" of the kernel with four lanes per (site, right-hand side), R = 1
 constexpr int PERS_DEFAULT_THREADS = 512;  // measured best at 32^3 x 8 (one and 16 right-hand sides)
 
 // Sites per tile for a phase whose blocks cover spb sites at a time: when the grid covers the
@@ -133,16 +135,19 @@ __device__ __forceinline__ int tile_sites(int count, int spb) {
 // tid = site_row * t + gi holds dot[r] of column gi * R + r (ndots = t * R columns).  With t a
 // power of two the lanes of one column meet in a shuffle tree and the warps' sums in one more
 // step; otherwise the dots go through red[rows][ndots] (red holds blockDim.x * R doubles).
-template <int R>
+// With S lanes per thread position (tid = (site_row * t + gi) * S + part) the dots are in part 0.
+template <int R, int S = 1>
 __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, double (&dot)[R], int t, int gi,
                                              int ndots, int col0 = 0) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int tS = t * S;
+    const bool own = S == 1 || tid % S == 0;
     __syncthreads();  // red may still be read by the previous step
-    if ((t & (t - 1)) == 0 && t <= 32) {
-        for (int off = 16; off >= t; off >>= 1)
+    if ((t & (t - 1)) == 0 && tS <= 32) {
+        for (int off = 16; off >= tS; off >>= 1)
 #pragma unroll
             for (int r = 0; r < R; r++) dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], off);
-        if (lane < t) {
+        if (lane < tS && own) {
 #pragma unroll
             for (int r = 0; r < R; r++)
                 if (gi * R + r < ndots) red[warp * ndots + gi * R + r] = dot[r];
@@ -156,10 +161,10 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, dou
         }
         return;
     }
-    const int rows = blockDim.x / t, row = tid / t;
+    const int rows = blockDim.x / tS, row = tid / tS;
     for (int i = tid; i < rows * ndots; i += blockDim.x) red[i] = 0.0;
     __syncthreads();
-    if (row < rows) {
+    if (row < rows && own) {
 #pragma unroll
         for (int r = 0; r < R; r++)
             if (gi * R + r < ndots) red[row * ndots + gi * R + r] = dot[r];
@@ -176,21 +181,22 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, dou
 
 // The same for K sets of dots in one pass: dot[k][r] is column k step + gi R + r (n = t R,
 // step >= n); red holds K blockDim.x * R doubles.
-template <int R, int K>
+template <int R, int K, int S = 1>
 __device__ __forceinline__ void publish_dots_k(const PersArgs &a, double *red, double (&dot)[K][R], int t, int gi,
                                                int n, int step) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    const int nd = K * n;
+    const int nd = K * n, tS = t * S;
+    const bool own = S == 1 || tid % S == 0;
     // set k, column j of the set, lands in partials column k * step + j
     auto column = [&](int jj) { return (jj / n) * step + jj % n; };
     __syncthreads();  // red may still be read by the previous step
-    if ((t & (t - 1)) == 0 && t <= 32) {
-        for (int off = 16; off >= t; off >>= 1)
+    if ((t & (t - 1)) == 0 && tS <= 32) {
+        for (int off = 16; off >= tS; off >>= 1)
 #pragma unroll
             for (int k = 0; k < K; k++)
 #pragma unroll
                 for (int r = 0; r < R; r++) dot[k][r] += __shfl_xor_sync(0xffffffffu, dot[k][r], off);
-        if (lane < t) {
+        if (lane < tS && own) {
 #pragma unroll
             for (int k = 0; k < K; k++)
 #pragma unroll
@@ -206,10 +212,10 @@ __device__ __forceinline__ void publish_dots_k(const PersArgs &a, double *red, d
         }
         return;
     }
-    const int rows = blockDim.x / t, row = tid / t;
+    const int rows = blockDim.x / tS, row = tid / tS;
     for (int i = tid; i < rows * nd; i += blockDim.x) red[i] = 0.0;
     __syncthreads();
-    if (row < rows) {
+    if (row < rows && own) {
 #pragma unroll
         for (int k = 0; k < K; k++)
 #pragma unroll
@@ -276,8 +282,10 @@ __device__ __forceinline__ void sum_partials(const PersArgs &a, double *red, int
 // (ax from the loader `ax` at the output site); with DOTS2 also |out|^2, published as columns
 // 2n..3n-1 (columns n..2n-1 are left to the update phase's |r|^2).  EPI_RESID (FP64):
 // r = b - m^2 ax + D in, written to out_lo (iterated precision Q) with |r|^2 per block.  mask[r]
-// selects right-hand sides; m2v[r] is the m^2 of right-hand side r (shared memory).
-template <int PP, int R, int EPI, int Q, class IN, class AX, bool DOTS2 = false>
+// selects right-hand sides; m2v[r] is the m^2 of right-hand side r (shared memory).  S = 4: four lanes
+// share a site and right-hand side (site_stencil's split), for lattices whose share per block leaves
+// most threads idle otherwise.
+template <int PP, int R, int EPI, int Q, class IN, class AX, bool DOTS2 = false, int S = 1>
 __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField &fat, const LinkField &naik,
                                              const IN &in, void *out, int parity, const int *mask, const AX &ax,
                                              const void *bvec, void *out_lo, double *red, const double *m2v,
@@ -286,8 +294,9 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
     const Geom &g = a.g;
     // with a list (R = 1), one thread per (site, listed right-hand side): a pass over u of the
     // bundle's n right-hand sides costs u / n of a full pass instead of idling n - u lanes
-    const int n = a.n, t = list ? nlist : n / R, spb = blockDim.x / t;
-    const int tid = threadIdx.x, gi = tid % t, sl = tid / t, r0 = list ? list[gi] : gi * R;
+    const int n = a.n, t = list ? nlist : n / R, spb = blockDim.x / (t * S);
+    const int tid = threadIdx.x, part = tid % S, gi = (tid / S) % t, sl = tid / (t * S);
+    const int r0 = list ? list[gi] : gi * R;
     const VecView<PP> vout{out, n};
     bool act[R];
     bool any = false;
@@ -302,11 +311,12 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
 #pragma unroll
         for (int r = 0; r < R; r++) dot[k][r] = 0.0;
     const int ts = tile_sites(g.Vh, spb);
-    if (any && sl < ts) {
+    if (S > 1 || (any && sl < ts)) {
         for (int tile = blockIdx.x; (long)tile * ts < g.Vh; tile += gridDim.x) {
             const int q = tile * ts + sl;
-            if (q >= g.Vh) break;
-            const int s = visit_site(g, q);
+            const bool valid = S == 1 || (any && sl < ts && q < g.Vh);
+            if (S == 1 && q >= g.Vh) break;
+            const int s = visit_site(g, valid ? q : 0);
             Cplx<real> acc[R][3];
             // 16-bit storage: the epilogue's own record (one 16-byte word per site and RHS) is
             // requested before the stencil, so its L2 latency overlaps the link and neighbour
@@ -315,7 +325,25 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
             uint4 raw = make_uint4(0, 0, 0, 0);
             if constexpr (EARLY)
                 if (act[0]) raw = __ldcg(reinterpret_cast<const uint4 *>(ax.v.data) + (size_t)s * n + r0);
-            site_stencil<PP, 18, R, 1>(g, fat, naik, parity, in, s, 0, r0, act, acc);
+            if constexpr (S == 1) {
+                site_stencil<PP, 18, R, 1>(g, fat, naik, parity, in, s, 0, r0, act, acc);
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; r++)
+#pragma unroll
+                    for (int c = 0; c < 3; c++) acc[r][c] = {0, 0};
+                if (valid) site_stencil<PP, 18, R, S>(g, fat, naik, parity, in, s, part, r0, act, acc);
+#pragma unroll
+                for (int off = 1; off < S; off <<= 1)  // every lane of the warp takes part
+#pragma unroll
+                    for (int r = 0; r < R; r++)
+#pragma unroll
+                        for (int c = 0; c < 3; c++) {
+                            acc[r][c].re += __shfl_xor_sync(0xffffffffu, acc[r][c].re, off);
+                            acc[r][c].im += __shfl_xor_sync(0xffffffffu, acc[r][c].im, off);
+                        }
+                if (!valid || part != 0) continue;
+            }
             if constexpr (EPI == EPI_PLAIN) {
                 store_adjacent<PP, R>(vout, s, r0, act, acc);
             } else if constexpr (EPI == EPI_AOP) {
@@ -373,9 +401,9 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
         }
     }
     if constexpr (DOTS2) {
-        publish_dots_k<R, 2>(a, red, dot, t, gi, n, 2 * n);
+        publish_dots_k<R, 2, S>(a, red, dot, t, gi, n, 2 * n);
     } else if constexpr (EPI != EPI_PLAIN) {
-        publish_dots<R>(a, red, dot[0], t, gi, list ? nlist : n);  // with a list: column i = list[i]
+        publish_dots<R, S>(a, red, dot[0], t, gi, list ? nlist : n);  // with a list: column i = list[i]
     }
 }
 
@@ -389,13 +417,14 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
 // EPI_PLAIN: out = D in (ds bundles).  EPI_RESID: r = b - m^2 x + D in with x, b FP64
 // and an FP64 epilogue, written to out_lo in the iterated precision Q, with |r|^2 per block
 // published as column i of the list.
-template <int EPI, int Q, int DR, bool PF>
+// S = 4: four lanes per (site, right-hand side), four links each, on small lattices (see dslash_phase).
+template <int EPI, int Q, int DR, bool PF, int S = 1>
 __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void *out, int parity, const void *xvec,
                                          const void *bvec, void *out_lo, double *red, const double *m2v,
                                          const int *list, int nlist) {
     const Geom &g = a.g;
-    const int n = a.n, t = (nlist + DR - 1) / DR, spb = blockDim.x / t;
-    const int tid = threadIdx.x, gi = tid % t, sl = tid / t;
+    const int n = a.n, t = (nlist + DR - 1) / DR, spb = blockDim.x / (t * S);
+    const int tid = threadIdx.x, part = tid % S, gi = (tid / S) % t, sl = tid / (t * S);
     bool act[DR];
     int rr[DR];
 #pragma unroll
@@ -407,14 +436,31 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
 #pragma unroll
     for (int r = 0; r < DR; r++) dot[r] = 0.0;
     const int ts = tile_sites(g.Vh, spb);
-    if (sl < ts) {
+    if (S > 1 || sl < ts) {
         for (int tile = blockIdx.x; (long)tile * ts < g.Vh; tile += gridDim.x) {
             const int q = tile * ts + sl;
-            if (q >= g.Vh) break;
-            const int s = visit_site(g, q);
+            const bool valid = S == 1 || (sl < ts && q < g.Vh);
+            if (S == 1 && q >= g.Vh) break;
+            const int s = visit_site(g, valid ? q : 0);
             dscplx acc[DR][3];
-            ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s, rr,
-                                          act, acc);
+            if constexpr (S == 1) {
+                ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
+                                              rr, act, acc);
+            } else {
+                static_assert(S == 4, "four lanes take four links each");
+                ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
+                                              rr, act, acc, 4 * part, valid ? 4 * part + 4 : 4 * part);
+#pragma unroll
+                for (int off = 1; off < S; off <<= 1)  // every lane of the warp takes part
+#pragma unroll
+                    for (int r = 0; r < DR; r++)
+#pragma unroll
+                        for (int c = 0; c < 3; c++) {
+                            acc[r][c].re = ds_add_lane(acc[r][c].re, off);
+                            acc[r][c].im = ds_add_lane(acc[r][c].im, off);
+                        }
+                if (!valid || part != 0) continue;
+            }
 #pragma unroll
             for (int r = 0; r < DR; r++) {
                 if (!act[r]) continue;
@@ -442,7 +488,7 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
             }
         }
     }
-    if constexpr (EPI == EPI_RESID) publish_dots<DR>(a, red, dot, t, gi, nlist);
+    if constexpr (EPI == EPI_RESID) publish_dots<DR, S>(a, red, dot, t, gi, nlist);
 }
 
 // x_hi of one site and right-hand side, written in double-single form for the recomputation
@@ -458,8 +504,8 @@ __device__ __forceinline__ void store_xds(const PersArgs &a, int s, int r, const
 }
 
 // the solve loop (body in cg_persistent_body.cuh, instantiated per precision)
-template <int P, int R, bool CG1>
-__global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const __grid_constant__ PersArgs a);
+template <int P, int R, bool CG1, int S>
+__global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(const __grid_constant__ PersArgs a);
 
 template <int P>
 cudaError_t launch_persistent_prec(const PersArgs &a, int R, bool cg1, int grid, int threads, size_t smem,

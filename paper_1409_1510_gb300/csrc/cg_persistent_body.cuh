@@ -4,8 +4,8 @@
 
 namespace hisq {
 
-template <int P, int R, bool CG1>
-__global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const __grid_constant__ PersArgs a) {
+template <int P, int R, bool CG1, int S>
+__global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(const __grid_constant__ PersArgs a) {
     constexpr int Q = q_prec(P);
     using rp = typename Prec<P>::real;
     using rq = typename Prec<Q>::real;
@@ -31,6 +31,14 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
 #define VQ(f) VecView<Q>{a.f, n}
 #define VP(f) VecView<P>{a.f, n}
     const bool row_ok = sl < ts;
+    // a Dslash phase of the iteration (out = D in, or A p's second half), and the two halves of a residual
+    // recomputation in double-single arithmetic
+#define DSLASH(EPI, DOTS2, f, out, parity)                                                                         \
+    dslash_phase<P, R, EPI, Q, PlainIn<P, true>, PlainIn<P, true>, DOTS2, S>(                                      \
+        a, a.fat, a.naik, PlainIn<P, true>{VP(f)}, out, parity, st.active, PlainIn<P, true>{VP(p)}, nullptr, nullptr, \
+        red, st.mass2)
+#define DS_PHASE(EPI, in, out, parity, x, b, lo) \
+    ds_phase<EPI, Q, 1, false, S>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n)
 
     // ---- setup: x_hi = 0, x = 0, r = b, p = b and |b|^2 ----
     {
@@ -70,13 +78,11 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
     // ---- Hestenes-Stiefel CG with one reduction: three phases an iteration ----
     while (CG1 && ok && st.any_active && st.bundle_iters < st.max_iter) {
         // t = D_oe p
-        dslash_phase<P, R, EPI_PLAIN, Q>(a, a.fat, a.naik, PlainIn<P, true>{VP(p)}, a.t, 1, st.active,
-                                         PlainIn<P, true>{VP(p)}, nullptr, nullptr, red, st.mass2);
+        DSLASH(EPI_PLAIN, false, p, a.t, 1);
         if (!(ok = grid_sync(a))) break;
         clock_mark(clk, PH_DOE);
         // A p = m^2 p - D_eo t with <p, A p> and |A p|^2 (|r|^2 came from the previous update phase)
-        dslash_phase<P, R, EPI_AOP, Q, PlainIn<P, true>, PlainIn<P, true>, true>(
-            a, a.fat, a.naik, PlainIn<P, true>{VP(t)}, a.ap, 0, st.active, PlainIn<P, true>{VP(p)}, nullptr, nullptr, red, st.mass2);
+        DSLASH(EPI_AOP, true, t, a.ap, 0);
         if (!(ok = grid_sync(a))) break;
         sum_partials(a, red, 3 * n, dots);
         if (tid == 0) run_hook(HOOK_CG1, &st, dots, n);
@@ -143,17 +149,17 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
             }
             __syncthreads();
             if constexpr (P == HISQ_FP64) {
-                dslash_phase<HISQ_FP64, 1, EPI_PLAIN, Q>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.t64,
+                dslash_phase<HISQ_FP64, 1, EPI_PLAIN, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.t64,
                                                          1, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, nullptr,
                                                          nullptr, red, st.mass2, upd_list, upd_n);
                 if (!(ok = grid_sync(a))) break;
-                dslash_phase<HISQ_FP64, 1, EPI_RESID, Q>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(t64)},
+                dslash_phase<HISQ_FP64, 1, EPI_RESID, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(t64)},
                                                          nullptr, 0, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.b,
                                                          a.r, red, st.mass2, upd_list, upd_n);
             } else {
-                ds_phase<EPI_PLAIN, Q, 1, false>(a, a.xds, a.t64, 1, nullptr, nullptr, nullptr, red, st.mass2, upd_list, upd_n);
+                DS_PHASE(EPI_PLAIN, a.xds, a.t64, 1, nullptr, nullptr, nullptr);
                 if (!(ok = grid_sync(a))) break;
-                ds_phase<EPI_RESID, Q, 1, false>(a, a.t64, nullptr, 0, a.xhi, a.b, a.r, red, st.mass2, upd_list, upd_n);
+                DS_PHASE(EPI_RESID, a.t64, nullptr, 0, a.xhi, a.b, a.r);
             }
             if (!(ok = grid_sync(a))) break;
             sum_partials(a, red, upd_n, dots);
@@ -184,13 +190,11 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
     // ---- Hestenes-Stiefel CG: four phases and two reductions an iteration ----
     while (!CG1 && ok && st.any_active && st.bundle_iters < st.max_iter) {
         // t = D_oe p
-        dslash_phase<P, R, EPI_PLAIN, Q>(a, a.fat, a.naik, PlainIn<P, true>{VP(p)}, a.t, 1, st.active,
-                                         PlainIn<P, true>{VP(p)}, nullptr, nullptr, red, st.mass2);
+        DSLASH(EPI_PLAIN, false, p, a.t, 1);
         if (!(ok = grid_sync(a))) break;
         clock_mark(clk, PH_DOE);
         // A p = m^2 p - D_eo t and <p, A p>
-        dslash_phase<P, R, EPI_AOP, Q>(a, a.fat, a.naik, PlainIn<P, true>{VP(t)}, a.ap, 0, st.active,
-                                       PlainIn<P, true>{VP(p)}, nullptr, nullptr, red, st.mass2);
+        DSLASH(EPI_AOP, false, t, a.ap, 0);
         if (!(ok = grid_sync(a))) break;
         sum_partials(a, red, n, dots);
         if (tid == 0) run_hook(HOOK_ALPHA, &st, dots, n);
@@ -251,11 +255,11 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
             }
             if (!(ok = grid_sync(a))) break;
             if constexpr (P == HISQ_FP64) {
-                dslash_phase<HISQ_FP64, 1, EPI_PLAIN, Q>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.t64,
+                dslash_phase<HISQ_FP64, 1, EPI_PLAIN, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.t64,
                                                          1, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, nullptr,
                                                          nullptr, red, st.mass2);
                 if (!(ok = grid_sync(a))) break;
-                dslash_phase<HISQ_FP64, 1, EPI_RESID, Q>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(t64)},
+                dslash_phase<HISQ_FP64, 1, EPI_RESID, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(t64)},
                                                          nullptr, 0, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.b,
                                                          a.r, red, st.mass2);
                 if (!(ok = grid_sync(a))) break;
@@ -270,9 +274,9 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
                     upd_n = u;
                 }
                 __syncthreads();
-                ds_phase<EPI_PLAIN, Q, 1, false>(a, a.xds, a.t64, 1, nullptr, nullptr, nullptr, red, st.mass2, upd_list, upd_n);
+                DS_PHASE(EPI_PLAIN, a.xds, a.t64, 1, nullptr, nullptr, nullptr);
                 if (!(ok = grid_sync(a))) break;
-                ds_phase<EPI_RESID, Q, 1, false>(a, a.t64, nullptr, 0, a.xhi, a.b, a.r, red, st.mass2, upd_list, upd_n);
+                DS_PHASE(EPI_RESID, a.t64, nullptr, 0, a.xhi, a.b, a.r);
                 if (!(ok = grid_sync(a))) break;
                 sum_partials(a, red, upd_n, dots);
                 if (tid == 0)
@@ -301,6 +305,8 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
         if (!(ok = grid_sync(a))) break;
         clock_mark(clk, PH_PUPDATE);
     }
+#undef DSLASH
+#undef DS_PHASE
 #undef V64
 #undef VQ
 #undef VP
@@ -314,15 +320,16 @@ __global__ void __launch_bounds__(pers_threads(R), 1) cg_persistent_kernel(const
     }
 }
 
-// the instantiation for R right-hand sides per thread (FP64 stops at two: four would spill) and
-// the CG form
+// the instantiation for R right-hand sides per thread (FP64 stops at two: four would spill; PERS_SPLIT:
+// four lanes per site and right-hand side) and the CG form
 template <int P, bool CG1>
 const void *persistent_kernel_ptr(int R) {
+    if (R == PERS_SPLIT) return (const void *)cg_persistent_kernel<P, 1, CG1, 4>;
     if constexpr (P != HISQ_FP64) {
-        if (R == 4) return (const void *)cg_persistent_kernel<P, 4, CG1>;
+        if (R == 4) return (const void *)cg_persistent_kernel<P, 4, CG1, 1>;
     }
-    if (R >= 2) return (const void *)cg_persistent_kernel<P, 2, CG1>;
-    return (const void *)cg_persistent_kernel<P, 1, CG1>;
+    if (R >= 2) return (const void *)cg_persistent_kernel<P, 2, CG1, 1>;
+    return (const void *)cg_persistent_kernel<P, 1, CG1, 1>;
 }
 
 template <int P>

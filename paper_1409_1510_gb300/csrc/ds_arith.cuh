@@ -49,6 +49,15 @@ __device__ __forceinline__ dsacc ds_normalize(dsacc s) {
     return {t, err};
 }
 
+// this lane's accumulator plus that of the lane `off` away: two-sum of the high parts, everything else low
+__device__ __forceinline__ dsacc ds_add_lane(dsacc s, int off) {
+    const float hi = __shfl_xor_sync(0xffffffffu, s.hi, off), lo = __shfl_xor_sync(0xffffffffu, s.lo, off);
+    const float t = __fadd_rn(s.hi, hi);
+    const float z = __fsub_rn(t, s.hi);
+    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, z)), __fsub_rn(hi, z));
+    return {t, __fadd_rn(__fadd_rn(s.lo, lo), err)};
+}
+
 __device__ __forceinline__ double ds_value(dsacc s) { return (double)s.hi + (double)s.lo; }
 
 __device__ __forceinline__ void ds_split(double x, float &hi, float &lo) {
@@ -131,11 +140,12 @@ struct DsOperands {
 // link are requested before the current one is applied, column by column (six independent
 // accumulation chains): twice the operand registers for more loads in flight (the recomputation
 // is bound by memory latency with one thread per site and right-hand side).  Without it (kernels
-// that must stay within 64 or 128 registers) each link row is requested just before its use.
+// that must stay within 64 or 128 registers) each link row is requested just before its use, and a lane
+// can take the links [k0, k1) only.
 template <int R, bool COHERENT, bool PREFETCH = false>
 __device__ __forceinline__ void ds_site_stencil(const Geom &g, const LinkField &fat, const LinkField &naik, int parity,
                                                 const float4 *in, int n, int s, const int rr[R], const bool act[R],
-                                                dscplx acc[R][3]) {
+                                                dscplx acc[R][3], int k0 = 0, int k1 = 16) {
     const SiteCoord sc = decode_site(g, s, parity);
 #pragma unroll
     for (int r = 0; r < R; r++)
@@ -156,7 +166,7 @@ __device__ __forceinline__ void ds_site_stencil(const Geom &g, const LinkField &
     } else {
         // few registers: each link's words are requested row by row, just before their use
 #pragma unroll 1
-        for (int k = 0; k < 16; k++) {
+        for (int k = k0; k < k1; k++) {
             const bool nk = k >= 8;
             const LinkField &f = nk ? naik : fat;
             const int slot = k & 7, hop = nk ? 3 : 1;

@@ -885,6 +885,13 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     // right-hand sides.  FP16 keeps four (its records unpack into packed pairs): 3% faster there.
     if ((S.prec == HISQ_FP32 || S.prec == HISQ_BF16) && R > 2) R = 2;
     while (S.n % R) R /= 2;
+    // a lattice so small that with one block per SM every site and right-hand side of a block's share gets
+    // four lanes, each applying four links in place of 16 (beyond that the lanes would take turns).  At
+    // 8^3 x 4 a block has seven sites: one lane each left 9200 cycles of FP64 multiply-adds in one chain of
+    // instructions with 25 lanes idle; plain FP64 CG there 3.20 -> 1.43 ms
+    const long share = (S.ctx->geom.Vh + S.ctx->num_sms - 1) / S.ctx->num_sms;
+    const bool split = S.ctx->params.persistent_threads == 0 && share * S.n * 4 <= PERS_DEFAULT_THREADS;
+    if (split) R = 1;
     // block size: the parameter if set (a multiple of 32 up to the kernel's bound), else 512
     int threads = std::min(pers_threads(R), PERS_DEFAULT_THREADS);
     const int want = S.ctx->params.persistent_threads;
@@ -892,10 +899,12 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     const size_t smem = (size_t)(4 * threads * R + 64) * sizeof(double);  // four dot sets (single reduction)
     int per_sm = 0;
     const bool cg1 = S.ctx->params.single_reduction != 0;
-    if (persistent_occ(S.prec, R, cg1, threads, smem, &per_sm) != cudaSuccess || per_sm < 1) {
+    const int kernel_R = split ? PERS_SPLIT : R;
+    if (persistent_occ(S.prec, kernel_R, cg1, threads, smem, &per_sm) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         return HISQ_OK;
     }
+    if (split) per_sm = 1;
     const int grid = per_sm * S.ctx->num_sms;  // one wave: every block resident (cooperative launch)
     if ((size_t)grid * PERS_ND > w->partials_cap) return HISQ_OK;
     PersArgs a;
@@ -943,7 +952,7 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
         HISQ_CUDA(cudaEventRecord(w->ev0, S.st));
     }
     const bool l2 = l2_window_begin(S.ctx, S.st, S.naik);
-    cudaError_t e = persistent_launch(S.prec, a, R, cg1, grid, threads, smem, S.st);
+    cudaError_t e = persistent_launch(S.prec, a, kernel_R, cg1, grid, threads, smem, S.st);
     if (l2) l2_window_end(S.st);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
         cudaGetLastError();

@@ -260,3 +260,18 @@ def test_reliable_update_threshold_by_precision():
             assert stats.converged == 2
             updates[delta] = stats.reliable_updates
         assert updates[0.0] <= updates[0.1], updates
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+@pytest.mark.parametrize("dims,n", [((4, 4, 4, 4), 1), ((4, 4, 4, 6), 5), ((8, 8, 8, 4), 3), ((8, 10, 8, 6), 9),
+                                    ((8, 10, 8, 6), 10)])
+def test_four_lanes_per_site_on_small_lattices(prec, dims, n):
+    """The persistent solve with four lanes per site and right-hand side: fewer sites than blocks, thread
+    positions that are no power of two, the last bundle it takes on 152 SMs (13 sites x 9) and the first
+    it does not; both CG forms, uneven norms."""
+    with gpu(dims, prec) as g:
+        rhs = [hi.gaussian_rhs(g.lat, 60 + k) * 10.0 ** (k % 4 - 2) for k in range(n)]
+        for single in (0, 1):
+            x, stats, iters, res = _solve(g, rhs, 0.1, inner_prec=prec, bundle=n, single_reduction=single)
+            true = g.oracle.true_residual(np.stack(rhs), x, 0.1)
+            assert np.all(true <= TOL * SLACK), (single, true)
