@@ -398,6 +398,7 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     a.axpy = d.axpy_in;
     a.b = d.b;
     a.b_one = d.b_one;
+    a.canon = d.canon;
     a.out_lo = d.out_lo;
     a.lo_prec = d.lo_prec;
     a.active = d.active;
@@ -602,6 +603,7 @@ int hisq_finalize(void) {
     }
     if (ctx->partials) cudaFree(ctx->partials);
     if (ctx->tmp) cudaFree(ctx->tmp);
+    if (ctx->resid) cudaFree(ctx->resid);
     if (ctx->counter) cudaFree(ctx->counter);
     if (ctx->dot_out) cudaFree(ctx->dot_out);
     if (ctx->dev_err) cudaFree(ctx->dev_err);

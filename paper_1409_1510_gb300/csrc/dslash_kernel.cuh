@@ -39,6 +39,7 @@ struct KArgs {
     const void *axpy;
     const void *b;
     int b_one;             // EPI_RESID: b is one right-hand side shared by the bundle
+    int canon;             // EPI_RESID, double-single: axpy, b and out are canonical [n][Vh][3] complex FP64
     void *out_lo;
     int lo_prec;
     const int *active;

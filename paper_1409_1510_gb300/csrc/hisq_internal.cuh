@@ -334,6 +334,8 @@ inline size_t staged_smem(int words_per_site, int TS, int threads, int n, bool r
     return 16 + (size_t)2 * words_per_site * TS * 16 + red;
 }
 
+constexpr size_t HISQ_RESID_KEEP = (size_t)1 << 30;
+
 struct Workspace;  // solver workspace (solver.cu)
 struct MsWork;     // multi-shift solver workspace (multishift.cu)
 
@@ -358,6 +360,9 @@ struct hisq_ctx {
     size_t tmp_cap;
     hisq::Workspace *ws;
     hisq::MsWork *ms = nullptr;
+    // scratch of hisq_residual, kept from call to call up to HISQ_RESID_KEEP bytes
+    char *resid = nullptr;
+    size_t resid_cap = 0;
     // L2 persisting set-aside for the link window of the persistent solve
     int l2_persist_max = -1, l2_window_max = 0;  // device limits (-1: not queried yet)
     bool l2_limit_saved = false;                 // l2_limit_old holds the context's limit before ours
@@ -397,6 +402,8 @@ struct DslashArgs {
     const void *axpy_in;   // EPI_AOP: p (same precision); EPI_RESID: x_hi (FP64)
     const void *b;         // EPI_RESID: right-hand side b (FP64 internal)
     int b_one;             // EPI_RESID: b holds one right-hand side, shared by all of the bundle
+    int canon;             // EPI_RESID in double-single arithmetic: axpy_in, b and out are canonical
+                           // double[n][Vh][3][2] (16-byte aligned) instead of internal bundles
     void *out_lo;          // EPI_RESID: sloppy copy of the new residual (lo_prec) or null
     int lo_prec;
     const int *active;     // per-rhs mask (null = all)
@@ -455,6 +462,8 @@ inline int copy_prec(const hisq_links *fat, int copy) {
 // (gs = g, t_off = 0: the whole lattice; otherwise one slab with ghost planes)
 void pack_links_into(int prec, int recon, const Geom &g, const Geom &gs, int t_off, int t_lo, int t_hi,
                      const double *U, int hop, uint4 *words, float *scale, int W, cudaStream_t st);
+// canonical double[n][Vh][3][2] (16-byte aligned) -> double-single bundle (dslash_ds.cu)
+int split_canonical(hisq_ctx *ctx, const double *canon, void *ds_bundle, int n, cudaStream_t st);
 // FP64 bundle -> double-single bundle of n right-hand sides (dslash_ds.cu)
 int split_vectors(hisq_ctx *ctx, const void *fp64_bundle, void *ds_bundle, int n, cudaStream_t st);
 void free_workspace(hisq_ctx *ctx);  // solver.cu

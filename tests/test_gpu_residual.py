@@ -49,3 +49,24 @@ def test_residual_at_convergence(prec):
         bn = np.linalg.norm(b)
         assert np.linalg.norm(r[0] - (b - g.oracle.aop(x, MASS))) <= 1e-12 * bn
         assert abs(np.sqrt(res2[0]) / bn - want) <= 0.01 * want
+
+
+@pytest.mark.parametrize("prec", [1, 2, 0])
+def test_device_buffers_read_and_written_in_place(prec):
+    """Device b, x, r at 16-byte addresses (used directly) and 8 bytes off (copied), calls of growing and
+    shrinking size on the kept scratch: bit for bit the result from host buffers."""
+    with gpu((8, 6, 4, 6), prec) as g:
+        for n in (1, 5, 2):
+            b = np.stack([hi.gaussian_rhs(g.lat, 400 + k) for k in range(n)])
+            x = np.stack([hi.gaussian_rhs(g.lat, 500 + k) for k in range(n)])
+            want, want2 = _residual(g, b, x)
+            size = b.size * 2
+            for ob, ox, orr in ((0, 0, 0), (1, 0, 0), (0, 1, 0), (0, 0, 1), (1, 1, 1)):
+                bufs = [g.torch.zeros(size + 2, dtype=g.torch.float64, device=g.dev)[o:o + size] for o in (ob, ox, orr)]
+                assert [t.data_ptr() % 16 for t in bufs] == [8 * o for o in (ob, ox, orr)]
+                bufs[0].copy_(g.torch.from_numpy(b.view(np.float64).reshape(-1).copy()))
+                bufs[1].copy_(g.torch.from_numpy(x.view(np.float64).reshape(-1).copy()))
+                res2 = g.torch.zeros(n, dtype=g.torch.float64, device=g.dev)
+                g.hisq.hisq_residual(g.fat, g.naik, MASS, *bufs, n, res2)
+                assert np.array_equal(bufs[2].cpu().numpy(), want.view(np.float64).reshape(-1)), (n, ob, ox, orr)
+                assert np.array_equal(res2.cpu().numpy(), want2)
