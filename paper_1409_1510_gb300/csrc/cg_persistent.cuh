@@ -449,7 +449,7 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
             } else {
                 static_assert(S == 4, "four lanes take four links each");
                 ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
-                                              rr, act, acc, 4 * part, valid ? 4 * part + 4 : 4 * part);
+                                              rr, act, acc, 2 * part, valid ? 2 * part + 2 : 2 * part);
 #pragma unroll
                 for (int off = 1; off < S; off <<= 1)  // every lane of the warp takes part
 #pragma unroll

@@ -108,17 +108,15 @@ __device__ __forceinline__ void ds_column_acc(const uint4 m[3], const float4 vb,
     }
 }
 
-// the 9 words of link `slot` of a ds record and the neighbour vectors it multiplies
+// the 9 words of one link of a ds record and the neighbour vectors it multiplies
 template <int R, bool COHERENT>
 struct DsOperands {
     uint4 m[9];        // entry (a, b) in word 3 a + b
     float4 v[R][3];
-    __device__ __forceinline__ void load(const Geom &g, const SiteCoord &sc, const LinkField &f, int hop, int parity,
-                                         int s, int slot, const float4 *in, int n, const int rr[R], const bool act[R]) {
-        const uint4 *base = f.words + ((size_t)parity * f.W + (size_t)slot * 9) * g.Vh + s;
+    __device__ __forceinline__ void load(const uint4 *words, size_t plane, int nb, const float4 *in, int n,
+                                         const int rr[R], const bool act[R]) {
 #pragma unroll
-        for (int j = 0; j < 9; j++) m[j] = __ldg(base + (size_t)j * g.Vh);
-        const int nb = neighbour_rt(g, sc, s, slot >> 1, (slot & 1) ? -hop : hop);
+        for (int j = 0; j < 9; j++) m[j] = __ldg(words + j * plane);
 #pragma unroll
         for (int r = 0; r < R; r++)
 #pragma unroll
@@ -138,66 +136,48 @@ struct DsOperands {
 // The stencil of Eq. (3) at output site s of parity `parity` in ds arithmetic for the R
 // right-hand sides rr[0..R) of the ds input bundle `in` (n right-hand sides): the 8 fat and 8 Naik
 // links of the site's gathered ds records (slot 2 mu forward, 2 mu + 1 the backward -U^dagger, as
-// in every other precision) times the neighbouring input vectors, summed into acc.  The 16 links
-// run as one sequence (fat slots 0..7, then Naik).  With PREFETCH the words and vectors of the next
-// link are requested before the current one is applied, column by column (six independent
-// accumulation chains): twice the operand registers for more loads in flight (the recomputation
-// is bound by memory latency with one thread per site and right-hand side).  Without it (kernels
-// that must stay within 64 or 128 registers) each link row is requested just before its use, and a lane
-// can take the links [k0, k1) only.
+// in every other precision) times the neighbouring input vectors, summed into acc.  The loop runs over
+// the eight (kind, direction) pairs, both hops of a direction per step, column by column (six
+// independent accumulation chains); without PREFETCH a lane can take the pairs [k0, k1) only.  With
+// PREFETCH the operands of each link are requested while the link before it is applied, in two sets of
+// registers that take turns (one set copied into the other after every link cost 48 moves beside 360
+// FP32 operations).  One link per step with its rows loaded just before their use against both hops of
+// a direction per step, all of a link's words at once: recomputations of the 64^3 x 16 solve 198 / 188 ms,
+// of the 32^3 x 8 single solve 1.24 / 0.98 ms.
 template <int R, bool COHERENT, bool PREFETCH = false>
 __device__ __forceinline__ void ds_site_stencil(const Geom &g, const LinkField &fat, const LinkField &naik, int parity,
                                                 const float4 *in, int n, int s, const int rr[R], const bool act[R],
-                                                dscplx acc[R][3], int k0 = 0, int k1 = 16) {
+                                                dscplx acc[R][3], int k0 = 0, int k1 = 8) {
     const SiteCoord sc = decode_site(g, s, parity);
+    const size_t plane = g.Vh;
 #pragma unroll
     for (int r = 0; r < R; r++)
 #pragma unroll
         for (int c = 0; c < 3; c++) acc[r][c] = {{0.f, 0.f}, {0.f, 0.f}};
+    // first word of the forward link of pair k; the backward one is nine planes on
+    auto words = [&](int k) {
+        const LinkField &f = k >= 4 ? naik : fat;
+        return f.words + ((size_t)parity * f.W + (size_t)(k & 3) * 18) * plane + s;
+    };
+    auto hop = [&](int k, int sign) { return neighbour_rt(g, sc, s, k & 3, k >= 4 ? 3 * sign : sign); };
     if constexpr (PREFETCH) {
-        DsOperands<R, COHERENT> cur, nxt;
-        cur.load(g, sc, fat, 1, parity, s, 0, in, n, rr, act);
+        DsOperands<R, COHERENT> fwd, bwd;
+        fwd.load(words(0), plane, hop(0, 1), in, n, rr, act);
 #pragma unroll 1
-        for (int k = 0; k < 16; k++) {
-            if (k + 1 < 16) {
-                const bool nk = k + 1 >= 8;
-                nxt.load(g, sc, nk ? naik : fat, nk ? 3 : 1, parity, s, (k + 1) & 7, in, n, rr, act);
-            }
-            cur.apply(acc);
-            cur = nxt;
+        for (int k = 0; k < 8; k++) {
+            bwd.load(words(k) + 9 * plane, plane, hop(k, -1), in, n, rr, act);
+            fwd.apply(acc);
+            if (k + 1 < 8) fwd.load(words(k + 1), plane, hop(k + 1, 1), in, n, rr, act);
+            bwd.apply(acc);
         }
     } else {
-        // few registers: each link's words are requested row by row, just before their use
 #pragma unroll 1
         for (int k = k0; k < k1; k++) {
-            const bool nk = k >= 8;
-            const LinkField &f = nk ? naik : fat;
-            const int slot = k & 7, hop = nk ? 3 : 1;
-            const uint4 *base = f.words + ((size_t)parity * f.W + (size_t)slot * 9) * g.Vh + s;
-            const int nb = neighbour_rt(g, sc, s, slot >> 1, (slot & 1) ? -hop : hop);
-            float4 v[R][3];
-#pragma unroll
-            for (int r = 0; r < R; r++)
-#pragma unroll
-                for (int c = 0; c < 3; c++)
-                    v[r][c] = act[r] ? ds_load<COHERENT>(in, ((long)nb * 3 + c) * n + rr[r]) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int a = 0; a < 3; a++) {
-                uint4 m[3];
-#pragma unroll
-                for (int b = 0; b < 3; b++) m[b] = __ldg(base + (size_t)(3 * a + b) * g.Vh);
-#pragma unroll
-                for (int r = 0; r < R; r++)
-#pragma unroll
-                    for (int b = 0; b < 3; b++) {
-                        const float mr_hi = __uint_as_float(m[b].x), mr_lo = __uint_as_float(m[b].y);
-                        const float mi_hi = __uint_as_float(m[b].z), mi_lo = __uint_as_float(m[b].w);
-                        ds_mac(acc[r][a].re, mr_hi, mr_lo, v[r][b].x, v[r][b].y);
-                        ds_mac(acc[r][a].re, -mi_hi, -mi_lo, v[r][b].z, v[r][b].w);
-                        ds_mac(acc[r][a].im, mr_hi, mr_lo, v[r][b].z, v[r][b].w);
-                        ds_mac(acc[r][a].im, mi_hi, mi_lo, v[r][b].x, v[r][b].y);
-                    }
-            }
+            DsOperands<R, COHERENT> op;
+            op.load(words(k), plane, hop(k, 1), in, n, rr, act);
+            op.apply(acc);
+            op.load(words(k) + 9 * plane, plane, hop(k, -1), in, n, rr, act);
+            op.apply(acc);
         }
     }
 }

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(256) ds_split_canon_kernel(int Vh, int n, cons
 }
 
 template <int R, int EPI>
-__global__ void __launch_bounds__(256) dslash_ds_kernel(KArgs a) {
+__global__ void __launch_bounds__(256, R == 1 ? 2 : 1) dslash_ds_kernel(KArgs a) {
     extern __shared__ double red[];
     if (a.gate && *a.gate == 0) return;
     const Geom &g = a.g;
