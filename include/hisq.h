@@ -104,7 +104,8 @@ const char *hisq_last_error(void);
  * or, for Naik links only, 13 (two rows of W plus c, where N = c W, W in SU(3)) or 9 (eight
  * SU(3) parameters plus c); 13 and 9 are exact only for links of that form (Sec. 2: Naik links
  * can be rebuilt from 9 or 13/14 reals; fat links cannot).  16-bit 18-real links carry one
- * float scale per site.  When prec != HISQ_FP64 the handle also keeps an FP64 copy, used by the
+ * float scale per site and are kept a second time in the order of the tensor-core kernel (if memory
+ * allows).  When prec != HISQ_FP64 the handle also keeps an FP64 copy, used by the
  * solvers' FP64 residual recomputation.  The input is not retained. */
 int hisq_links_create(hisq_links **h, const double *canon, int is_naik, int prec, int recon);
 int hisq_links_destroy(hisq_links *h);
@@ -153,9 +154,8 @@ int hisq_aop(const hisq_links *fat, const hisq_links *naik, double mass, const v
  * exact products (Dekker 1971, by fused multiply-add) and error-free sums (Knuth's two-sum,
  * Ogita-Rump-Oishi cascaded summation) on the FP32 pipe, then b - m^2 x + D t in FP64; for FP64
  * handles native FP64.  rhs, x, r: host or device canonical double[nrhs][V/2][3][2] (r may alias
- * neither); res2: host or device double[nrhs] receiving |r_k|^2 (may be NULL).  Its scratch is
- * kept in the context (cudaMalloc when it grows) up to 1 GiB, released by hisq_finalize; a larger
- * one is allocated for the call.  Synchronises the context's stream. */
+ * neither); res2: host or device double[nrhs] receiving |r_k|^2 (may be NULL).  Allocates its
+ * scratch (cudaMalloc) for the call and synchronises the context's stream. */
 int hisq_residual(const hisq_links *fat, const hisq_links *naik, double mass, const double *rhs,
                   const double *x, double *r, int nrhs, double *res2);
 
@@ -357,9 +357,8 @@ int hisq_last_stats(hisq_solve_stats *s, int *iterations, double *true_residual)
  * precision, timing every candidate with CUDA events after an L2 flush.  Writes the
  * chosen right-hand sides per thread, threads per block and lanes per site (1; 2 when the fat
  * and Naik halves of a site run on two lanes; 4 when each lane takes two directions of one kind;
- * 8 for that split with staged link records, see hisq_set_launch_shape) if the pointers are not
- * NULL.  Allocates its
- * timing buffers. */
+ * 8 for that split with staged link records, 32 for the tensor-core kernel, see
+ * hisq_set_launch_shape) if the pointers are not NULL.  Allocates its timing buffers. */
 int hisq_autotune(const hisq_links *fat, const hisq_links *naik, int nrhs, int *rhs_per_thread,
                   int *block_threads, int *lanes_per_site);
 
@@ -368,7 +367,9 @@ int hisq_autotune(const hisq_links *fat, const hisq_links *naik, int nrhs, int *
  * lanes_per_site 1, 2 (18-real Naik links, rhs_per_thread <= 4) or 4 (18-real Naik links,
  * rhs_per_thread <= 2), or 8: the four-lane split with each tile's link records staged in shared
  * memory by the bulk-copy engine (18-real Naik, FP32/FP16/BF16, rhs_per_thread <= 2; tiles of
- * block_threads / (4 nrhs / rhs_per_thread) sites, block_threads up to 512).
+ * block_threads / (4 nrhs / rhs_per_thread) sites, block_threads up to 512), or 32: one warp per site
+ * on the tensor cores (18-real Naik, FP16 or BF16, 2..32 right-hand sides, an even number for BF16,
+ * rhs_per_thread 1; block_threads = 32 times the 1..32 sites of a row that a warp visits in one go).
  * Overrides the autotuner's choice for that key. */
 int hisq_set_launch_shape(int prec, int recon, int nrhs, int rhs_per_thread, int block_threads,
                           int lanes_per_site);

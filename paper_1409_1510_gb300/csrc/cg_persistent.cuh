@@ -14,6 +14,7 @@
 #pragma once
 #include "dslash_kernel.cuh"
 #include "ds_arith.cuh"
+#include "dslash_mma.cuh"
 
 namespace hisq {
 
@@ -26,6 +27,8 @@ struct PersArgs {
     void *x, *r;              // x_lo and r in the iterated precision
     void *b, *xhi, *t64;      // FP64 (t64: double-single when P != FP64)
     void *xds;                // x_hi in double-single form (P != FP64)
+    MmaField mfat, mnaik;     // the links' tensor-core copies (R = MMA_GROUP)
+    int run;                  // sites per warp's run of the tensor-core phases
     int n;
     double *partials;         // [gridDim][PERS_ND]
     SolverState *st;          // initial state in, final state out (block 0)
@@ -117,8 +120,8 @@ __device__ __forceinline__ bool grid_sync(const PersArgs &a) {
 }
 
 // Largest block: 1024 threads at one right-hand side per thread (64 registers), 512 otherwise
-// or with four lanes per site (128 registers); the launch may use fewer (a multiple of 32 dividing into
-// the SM's resources).
+// or with four lanes per site or the tensor-core phases (128 registers); the launch may use fewer (a
+// multiple of 32 dividing into the SM's resources).
 __host__ __device__ constexpr int pers_threads(int R, int S = 1) { return R == 1 && S == 1 ? 1024 : 512; }
 constexpr int PERS_SPLIT = -4;  // "R" of the kernel with four lanes per (site, right-hand side), R = 1
 constexpr int PERS_DEFAULT_THREADS = 512;  // measured best at 32^3 x 8 (one and 16 right-hand sides)
@@ -404,6 +407,66 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
         publish_dots_k<R, 2, S>(a, red, dot, t, gi, n, 2 * n);
     } else if constexpr (EPI != EPI_PLAIN) {
         publish_dots<R, S>(a, red, dot[0], t, gi, list ? nlist : n);  // with a list: column i = list[i]
+    }
+}
+
+// One Dslash phase on the tensor cores (dslash_mma.cuh), 16-bit storage, n <= MMA_GROUP: EPI_PLAIN or
+// EPI_AOP as in dslash_phase, every right-hand side of the bundle whether active or not (the rows of a
+// product cost the same; the masked ones' vectors and dots are not used).
+template <int PP, int N, int U, int EPI, bool DOTS2>
+__device__ __forceinline__ void mma_phase_n(const PersArgs &a, const void *in, void *out, int parity, const void *ax,
+                                            double *red, const double *m2v) {
+    const Geom &g = a.g;
+    const int n = N ? N : a.n;
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int nw = blockDim.x >> 5;
+    const MmaLane<PP, N> L(lane, n, 0);
+    const MmaRuns R = mma_runs(g, g.Vh, a.run);
+    float m2_lo = 0.f, m2_hi = 0.f;
+    if constexpr (EPI == EPI_AOP) {
+        m2_lo = (float)m2v[min(L.r_lo, n - 1)];
+        m2_hi = (float)m2v[min(L.r_hi, n - 1)];
+    }
+    const char *vin = mma_ptr(L, in), *vout = mma_ptr(L, out), *vax = mma_ptr(L, ax);
+    double sum = 0.0;  // lane q of a quad: Re <p, w> of the two right-hand sides, |w|^2 of the two
+    for (int u = blockIdx.x * nw + warp; u < R.count; u += gridDim.x * nw) {
+        MmaRun run;
+        if (!mma_run(g, R, u, parity, run)) continue;
+        mma_run_sites<PP, N, U, true>(g, a.mfat, a.mnaik, L, run, parity, vin, [&](int s, MmaC &w) {
+            if constexpr (EPI == EPI_AOP) {
+                float d[4];
+                mma_aop<PP, N, true>(L, vax, s, m2_lo, m2_hi, w, d);
+                sum += (double)mma_quad_sums(d, L.q);
+            }
+            mma_store(L, vout, s, w, L.has_lo, L.has_hi);
+        });
+    }
+    if constexpr (EPI == EPI_AOP) {
+        __syncthreads();  // red may still be read by the previous step
+        red[warp * 32 + lane] = sum;
+        __syncthreads();
+        for (int col = warp; col < 32; col += nw) {  // one lane position per warp: a shuffle tree over the warps
+            double s = lane < nw ? red[lane * 32 + col] : 0.0;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            const MmaLane<PP, N> C(col, n, 0);
+            const int r = (col & 1) ? C.r_hi : C.r_lo, dots2 = (col >> 1) & 1;
+            if (lane == 0 && r < n && (DOTS2 || !dots2))
+                a.partials[(size_t)blockIdx.x * PERS_ND + dots2 * 2 * n + r] = s;
+        }
+    }
+}
+
+template <int PP, int EPI, bool DOTS2 = false>
+__device__ __forceinline__ void mma_phase(const PersArgs &a, const void *in, void *out, int parity, const void *ax,
+                                          double *red, const double *m2v) {
+    if (mma_u(a.g.half) == 4) {
+        if (mma_n<PP>(a.n) == 16) mma_phase_n<PP, 16, 4, EPI, DOTS2>(a, in, out, parity, ax, red, m2v);
+        else mma_phase_n<PP, 0, 4, EPI, DOTS2>(a, in, out, parity, ax, red, m2v);
+    } else if (mma_u(a.g.half) == 2) {
+        mma_phase_n<PP, 0, 2, EPI, DOTS2>(a, in, out, parity, ax, red, m2v);
+    } else {
+        mma_phase_n<PP, 0, 1, EPI, DOTS2>(a, in, out, parity, ax, red, m2v);
     }
 }
 

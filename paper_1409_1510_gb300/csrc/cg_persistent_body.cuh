@@ -78,11 +78,17 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
     // ---- Hestenes-Stiefel CG with one reduction: three phases an iteration ----
     while (CG1 && ok && st.any_active && st.bundle_iters < st.max_iter) {
         // t = D_oe p
-        DSLASH(EPI_PLAIN, false, p, a.t, 1);
+        if constexpr (R == MMA_GROUP)
+            mma_phase<P, EPI_PLAIN>(a, a.p, a.t, 1, nullptr, red, st.mass2);
+        else
+            DSLASH(EPI_PLAIN, false, p, a.t, 1);
         if (!(ok = grid_sync(a))) break;
         clock_mark(clk, PH_DOE);
         // A p = m^2 p - D_eo t with <p, A p> and |A p|^2 (|r|^2 came from the previous update phase)
-        DSLASH(EPI_AOP, true, t, a.ap, 0);
+        if constexpr (R == MMA_GROUP)
+            mma_phase<P, EPI_AOP, true>(a, a.t, a.ap, 0, a.p, red, st.mass2);
+        else
+            DSLASH(EPI_AOP, true, t, a.ap, 0);
         if (!(ok = grid_sync(a))) break;
         sum_partials(a, red, 3 * n, dots);
         if (tid == 0) run_hook(HOOK_CG1, &st, dots, n);
@@ -190,11 +196,17 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
     // ---- Hestenes-Stiefel CG: four phases and two reductions an iteration ----
     while (!CG1 && ok && st.any_active && st.bundle_iters < st.max_iter) {
         // t = D_oe p
-        DSLASH(EPI_PLAIN, false, p, a.t, 1);
+        if constexpr (R == MMA_GROUP)
+            mma_phase<P, EPI_PLAIN>(a, a.p, a.t, 1, nullptr, red, st.mass2);
+        else
+            DSLASH(EPI_PLAIN, false, p, a.t, 1);
         if (!(ok = grid_sync(a))) break;
         clock_mark(clk, PH_DOE);
         // A p = m^2 p - D_eo t and <p, A p>
-        DSLASH(EPI_AOP, false, t, a.ap, 0);
+        if constexpr (R == MMA_GROUP)
+            mma_phase<P, EPI_AOP>(a, a.t, a.ap, 0, a.p, red, st.mass2);
+        else
+            DSLASH(EPI_AOP, false, t, a.ap, 0);
         if (!(ok = grid_sync(a))) break;
         sum_partials(a, red, n, dots);
         if (tid == 0) run_hook(HOOK_ALPHA, &st, dots, n);
@@ -321,10 +333,14 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
 }
 
 // the instantiation for R right-hand sides per thread (FP64 stops at two: four would spill; PERS_SPLIT:
-// four lanes per site and right-hand side) and the CG form
+// four lanes per site and right-hand side; MMA_GROUP: the tensor-core phases of 16-bit storage) and the
+// CG form
 template <int P, bool CG1>
 const void *persistent_kernel_ptr(int R) {
     if (R == PERS_SPLIT) return (const void *)cg_persistent_kernel<P, 1, CG1, 4>;
+    if constexpr (P == HISQ_FP16 || P == HISQ_BF16) {
+        if (R == MMA_GROUP) return (const void *)cg_persistent_kernel<P, MMA_GROUP, CG1, 1>;
+    }
     if constexpr (P != HISQ_FP64) {
         if (R == 4) return (const void *)cg_persistent_kernel<P, 4, CG1, 1>;
     }

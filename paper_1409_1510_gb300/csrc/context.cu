@@ -252,6 +252,36 @@ void pack_links_into(int prec, int recon, const Geom &g, const Geom &gs, int t_o
     }
 }
 
+// The tensor-core copy of a 16-bit 18-real field: word ((p Vh + s) 2 + j) 9 + e holds entry e = 3 a + b of
+// links 4 j .. 4 j + 3 (their re, im pairs as stored; BF16: half of those of column b = 0, which two lanes
+// of the kernel apply).  One thread per (site, j).
+__global__ void fragment_links_kernel(int Vh, const uint4 *words, uint4 *frag, bool bf16) {
+    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (i >= 4L * Vh) return;
+    const int j = (int)(i & 1);
+    const long site = i >> 1, parity = site / Vh, s = site - parity * Vh;  // site = parity Vh + s
+    uint32_t u[4][9];  // [link][entry]: 36 bytes per link, 9 words of 16 bytes for the four
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+        const uint4 w = words[((size_t)parity * 18 + 9 * j + k) * Vh + s];
+        const uint32_t v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int c = 0; c < 4; c++) u[(4 * k + c) / 9][(4 * k + c) % 9] = v[c];
+    }
+    if (bf16) {
+        const __nv_bfloat162 h = __float2bfloat162_rn(0.5f);
+#pragma unroll
+        for (int l = 0; l < 4; l++)
+#pragma unroll
+            for (int e = 0; e < 9; e += 3) {
+                const __nv_bfloat162 x = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(&u[l][e]), h);
+                u[l][e] = *reinterpret_cast<const uint32_t *>(&x);
+            }
+    }
+#pragma unroll
+    for (int e = 0; e < 9; e++) frag[(size_t)i * 9 + e] = make_uint4(u[0][e], u[1][e], u[2][e], u[3][e]);
+}
+
 static void dispatch_pack(int prec, int recon, const Geom &g, const double *U, int hop, uint4 *words, float *scale,
                           int W, cudaStream_t st) {
     pack_links_into(prec, recon, g, g, 0, 0, g.L[3], U, hop, words, scale, W, st);
@@ -331,6 +361,19 @@ LaunchShape default_shape(int prec, int n) {
 }
 
 
+// Whether the tensor-core kernel can take bundles of n with these links: 16-bit ones with their fragment
+// copies, 2 .. 32 right-hand sides, an even number for BF16 (whose lanes move two adjacent ones).
+bool mma_fields(const hisq_links *fat, const hisq_links *naik, int n) {
+    return fat->frag && naik->frag && n >= 2 && n <= MMA_MAX_N && (fat->prec == HISQ_FP16 || n % 2 == 0);
+}
+
+// And this launch: a whole parity of the context's lattice, buffers aligned to its 4- or 8-byte words.
+static bool mma_applies(const hisq_links *fat, const hisq_links *naik, int copy, const DslashArgs &d) {
+    const uintptr_t at = (uintptr_t)d.in | (uintptr_t)d.out | (uintptr_t)d.axpy_in;
+    return copy == LINKS_INNER && !d.geom && !d.fields && d.epi != EPI_RESID && d.site_end == 0 &&
+           mma_fields(fat, naik, d.n) && at % (fat->prec == HISQ_FP16 ? 4 : 8) == 0;
+}
+
 int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, int copy, const DslashArgs &d,
                   const LaunchShape *shape, cudaStream_t stream, int *grid_out) {
     if (copy == LINKS_DS && !fat->residual_ds()) copy = LINKS_FP64;  // FP64 handles have no ds copy
@@ -344,6 +387,8 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
         return set_error(HISQ_ERR_ARG, "a Dslash on another lattice needs its geometry, links and launch shape");
     const Geom &G = d.geom ? *d.geom : ctx->geom;
     LaunchShape sh = shape ? *shape : tuned_shape(ctx, fat, naik, d.n, copy);
+    const bool mma = sh.S == 32 && mma_applies(fat, naik, copy, d);
+    if (sh.S == 32 && !mma) sh = default_shape(prec, d.n);  // buffers or links that kernel cannot take
     int R = sh.R;
     if (R != 1 && R != 2 && R != 4 && R != 8) R = 1;
     if (d.n % R != 0) R = 1;
@@ -362,13 +407,18 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     if (!ds && recon == 18 && sh.S == 2 && R <= 4) S = 2;
     if (!ds && recon == 18 && sh.S == 4 && R <= 2) S = 4;
     const bool ranged = d.site_end > 0;  // the staged kernel covers whole parities only
+    if (mma) S = 32;
     if (!ds && !ranged && recon == 18 && sh.S == 8 && R <= 2 && prec != HISQ_FP64 && d.epi != EPI_RESID) S = 8;
     if (!ds && ranged && recon == 18 && sh.S == 8 && R <= 2) S = 4;
     int t = (d.n + R - 1) / R;
     // reducing epilogues finish in one block that sums a partial per block: blocks of at least 128
     // threads keep both the partial count and that block's share of the sum small
     int spb, threads;
-    if (S == 8) {
+    if (S == 32) {
+        t = (d.n + MMA_GROUP - 1) / MMA_GROUP;
+        spb = std::max(1, sh.threads / 32);  // sites per run
+        threads = MMA_THREADS;
+    } else if (S == 8) {
         // staged: threads = 4 t TS exactly (TS sites per tile), up to 512
         spb = std::max(1, std::min(sh.threads, 512) / (4 * t));
         threads = 4 * t * spb;
@@ -420,7 +470,14 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     }
 
     size_t smem = 0;
-    if (S == 8) {
+    if (S == 32) {
+        if (d.epi != EPI_PLAIN) {
+            smem = std::max((size_t)(MMA_THREADS / 32) * d.n, (size_t)threads + 64) * sizeof(double);
+            a.max_grid = (int)std::min<size_t>(d.partials_cap / d.n, 1u << 30);
+            if (!d.partials || !d.counter || a.max_grid < 1)
+                return set_error(HISQ_ERR_ARG, "reduction scratch too small for the Dslash epilogue");
+        }
+    } else if (S == 8) {
         smem = staged_smem(a.fat.W + a.naik.W, spb, threads, d.n, d.epi != EPI_PLAIN);
         if (smem > 227 * 1024)
             return set_error(HISQ_ERR_ARG, "staged launch shape needs %zu bytes of shared memory", smem);
@@ -440,7 +497,13 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     }
     int grid = 0;
     cudaError_t e;
-    switch (prec) {
+    if (S == 32)
+        e = prec == HISQ_FP16
+                ? launch_dslash_mma<HISQ_FP16>(a, {fat->frag, fat->scale}, {naik->frag, naik->scale}, d.epi, smem,
+                                               ctx->num_sms, stream, &grid)
+                : launch_dslash_mma<HISQ_BF16>(a, {fat->frag, fat->scale}, {naik->frag, naik->scale}, d.epi, smem,
+                                               ctx->num_sms, stream, &grid);
+    else switch (prec) {
     case HISQ_DS: e = launch_dslash_ds(a, d.epi, R, threads, smem, ctx->num_sms, stream, &grid); break;
     case HISQ_FP64: e = launch_dslash_prec<HISQ_FP64>(a, recon, d.epi, R, S, threads, smem, ctx->num_sms, stream, &grid); break;
     case HISQ_FP32: e = launch_dslash_prec<HISQ_FP32>(a, recon, d.epi, R, S, threads, smem, ctx->num_sms, stream, &grid); break;
@@ -573,6 +636,7 @@ int hisq_links_destroy(hisq_links *h) {
     if (h->scale) cudaFree(h->scale);
     if (h->words64) cudaFree(h->words64);
     if (h->words_ds) cudaFree(h->words_ds);
+    if (h->frag) cudaFree(h->frag);
     hisq_ctx *ctx = h->ctx;
     if (ctx) {
         ctx->links.erase(std::remove(ctx->links.begin(), ctx->links.end(), h), ctx->links.end());
@@ -647,6 +711,16 @@ int hisq_links_create(hisq_links **out, const double *canon, int is_naik, int pr
         cudaMalloc(&h->scale, (size_t)2 * g.Vh * sizeof(float)) != cudaSuccess)
         rc = set_error(HISQ_ERR_NOMEM, "cannot allocate link scales");
     if (rc == HISQ_OK) dispatch_pack(prec, recon, g, U, hop, h->words, h->scale, h->W, st);
+    if (rc == HISQ_OK && prec >= HISQ_FP16 && recon == 18) {
+        // the tensor-core copy; without memory for it the other kernels serve the field
+        if (cudaMalloc(&h->frag, wbytes) == cudaSuccess) {
+            fragment_links_kernel<<<(int)((4L * g.Vh + 127) / 128), 128, 0, st>>>(g.Vh, h->words, h->frag,
+                                                                                prec == HISQ_BF16);
+        } else {
+            cudaGetLastError();
+            h->frag = nullptr;
+        }
+    }
     if (rc == HISQ_OK && prec != HISQ_FP64) {
         // the FP64 copy (plain FP64 solves with these links) and the double-single copy (the
         // residual recomputations of mixed-precision solves)

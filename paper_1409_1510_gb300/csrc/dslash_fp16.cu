@@ -11,4 +11,11 @@ cudaError_t launch_dslash_prec<HISQ_FP16>(const KArgs &a, int recon, int epi, in
     return launch_epi<HISQ_FP16, 18>(a, epi, R, S, threads, smem, num_sms, s, grid);
 }
 
+template <>
+cudaError_t launch_dslash_mma<HISQ_FP16>(const KArgs &a, const MmaField &fat, const MmaField &naik, int epi, size_t smem,
+                                         int num_sms, cudaStream_t s, int *grid) {
+    if (epi == EPI_PLAIN) return launch_mma_one<HISQ_FP16, EPI_PLAIN>(a, fat, naik, smem, num_sms, s, grid);
+    return launch_mma_one<HISQ_FP16, EPI_AOP>(a, fat, naik, smem, num_sms, s, grid);
+}
+
 }  // namespace hisq

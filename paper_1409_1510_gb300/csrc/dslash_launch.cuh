@@ -3,6 +3,7 @@
 // translation unit so the instantiations compile in parallel.
 #pragma once
 #include "dslash_kernel.cuh"
+#include "dslash_mma.cuh"
 
 namespace hisq {
 
@@ -90,6 +91,12 @@ inline cudaError_t launch_epi(const KArgs &a, int epi, int R, int S, int threads
     }
     return launch_r<P, NR, EPI_AOP>(a, R, S, threads, smem, num_sms, s, grid);
 }
+
+// The tensor-core kernel (dslash_mma.cuh; defined in dslash_fp16.cu and dslash_bf16.cu), EPI_PLAIN or
+// EPI_AOP: a.t groups of right-hand sides, a.spb sites per run.
+template <int P>
+cudaError_t launch_dslash_mma(const KArgs &a, const MmaField &fat, const MmaField &naik, int epi, size_t smem,
+                              int num_sms, cudaStream_t s, int *grid);
 
 // The per-precision entry (defined in dslash_<prec>.cu).
 template <int P>

@@ -286,6 +286,8 @@ struct hisq_links {
     float *scale;          // [2][Vh] or null
     uint4 *words64;        // FP64 recon-18 copy (null when prec == FP64: use words)
     uint4 *words_ds;       // double-single recon-18 copy (null when prec == FP64)
+    uint4 *frag;           // 16-bit recon-18 records again, in the order of the tensor-core Dslash
+                           // (dslash_mma.cuh), or null (then that path is not taken)
     hisq::LinkField field() const { return {words, scale, W}; }
     hisq::LinkField field64() const {
         if (prec == HISQ_FP64 && recon == 18) return {words, nullptr, W};
@@ -324,7 +326,9 @@ struct LaunchShape {
     int threads;  // threads per block
     int S = 1;    // lanes per (site, rhs group): 2 splits the fat and Naik halves, 4 two directions
                   // of one kind per lane (18-real Naik); 8 = the 4-lane split with the tile's link
-                  // records staged in shared memory by the bulk-copy engine
+                  // records staged in shared memory by the bulk-copy engine; 32 = one warp per site on
+                  // the tensor cores (16-bit storage, 18-real Naik, 2..32 RHS, an even number
+                  // for BF16; R = 1; threads = sites of a row that a warp visits in one go, times 32)
 };
 
 // shared memory of the staged kernel for TS sites per tile: two stages of link records, the
@@ -447,6 +451,8 @@ inline size_t dslash_partials_needed(long Vh, int num_sms, int spb, int n) {
 }
 // (fat, naik) handles of this context with matching precisions (context.cu)
 int check_pair(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik);
+// whether the tensor-core Dslash can take bundles of n with these links (context.cu)
+bool mma_fields(const hisq_links *fat, const hisq_links *naik, int n);
 // grid_out (optional) receives the number of blocks launched (= partials written per dot)
 int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, int copy,
                   const DslashArgs &a, const LaunchShape *shape, cudaStream_t stream, int *grid_out = nullptr);

@@ -795,8 +795,8 @@ static int build_graph(const Solve &S) {
 // other field and the vectors stream from HBM.  The
 // set-aside is reserved once per context (restored by hisq_finalize) and the persisting lines are
 // released after each solve, so no solve starts with links left in L2 by another.
-static bool l2_window_begin(hisq_ctx *ctx, cudaStream_t st, const hisq_links *links) {
-    if (!ctx->params.l2_persist_links || !links->words) return false;
+static bool l2_window_begin(hisq_ctx *ctx, cudaStream_t st, const hisq_links *links, const uint4 *words) {
+    if (!ctx->params.l2_persist_links || !words) return false;
     if (ctx->l2_persist_max < 0) {
         int maxp = 0, maxw = 0;
         if (cudaDeviceGetAttribute(&maxp, cudaDevAttrMaxPersistingL2CacheSize, ctx->device) != cudaSuccess ||
@@ -831,7 +831,7 @@ static bool l2_window_begin(hisq_ctx *ctx, cudaStream_t st, const hisq_links *li
     }
     cudaStreamAttrValue v;
     memset(&v, 0, sizeof(v));
-    v.accessPolicyWindow.base_ptr = (void *)links->words;
+    v.accessPolicyWindow.base_ptr = (void *)words;  // the copy that the solve reads
     v.accessPolicyWindow.num_bytes = std::min(bytes, (size_t)ctx->l2_window_max);
     v.accessPolicyWindow.hitRatio = std::min(1.0f, (float)carve / (float)v.accessPolicyWindow.num_bytes);
     v.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
@@ -892,11 +892,14 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     const long share = (S.ctx->geom.Vh + S.ctx->num_sms - 1) / S.ctx->num_sms;
     const bool split = S.ctx->params.persistent_threads == 0 && share * S.n * 4 <= PERS_DEFAULT_THREADS;
     if (split) R = 1;
+    // the tensor-core phases where the tuner found that kernel the fastest for this bundle
+    const bool mma = !split && sh.S == 32 && S.prec != HISQ_FP64 && S.n <= MMA_GROUP && mma_fields(S.fat, S.naik, S.n);
+    if (mma) R = MMA_GROUP;
     // block size: the parameter if set (a multiple of 32 up to the kernel's bound), else 512
     int threads = std::min(pers_threads(R), PERS_DEFAULT_THREADS);
     const int want = S.ctx->params.persistent_threads;
     if (want >= 32 && want <= pers_threads(R) && want % 32 == 0) threads = want;
-    const size_t smem = (size_t)(4 * threads * R + 64) * sizeof(double);  // four dot sets (single reduction)
+    const size_t smem = (size_t)(4 * threads * (mma ? 1 : R) + 64) * sizeof(double);  // four dot sets (single reduction)
     int per_sm = 0;
     const bool cg1 = S.ctx->params.single_reduction != 0;
     const int kernel_R = split ? PERS_SPLIT : R;
@@ -922,6 +925,11 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
         a.fat64 = S.fat->field_ds();
         a.naik64 = S.naik->field_ds();
         a.xds = w->x_ds;
+    }
+    if (mma) {
+        a.mfat = {S.fat->frag, S.fat->scale};
+        a.mnaik = {S.naik->frag, S.naik->scale};
+        a.run = mma_run_length(a.g, a.g.Vh, (long)grid * (threads / 32));
     }
     a.p = w->p;
     a.t = w->t;
@@ -951,7 +959,7 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
         HISQ_CUDA(cudaMemsetAsync(w->phase_ns, 0, sizeof(unsigned long long) * 8, S.st));
         HISQ_CUDA(cudaEventRecord(w->ev0, S.st));
     }
-    const bool l2 = l2_window_begin(S.ctx, S.st, S.naik);
+    const bool l2 = l2_window_begin(S.ctx, S.st, S.naik, mma ? S.naik->frag : S.naik->words);
     cudaError_t e = persistent_launch(S.prec, a, kernel_R, cg1, grid, threads, smem, S.st);
     if (l2) l2_window_end(S.st);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {

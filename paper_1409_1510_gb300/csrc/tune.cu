@@ -94,6 +94,17 @@ static int run_tuner(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *nai
         }
         if (rc != HISQ_OK) break;
     }
+    // the tensor-core kernel, runs of 32, 16, 8 and 4 sites
+    if (copy == LINKS_INNER && mma_fields(fat, naik, n))
+        for (int run = 32; run >= 4 && rc == HISQ_OK; run /= 2) {
+            LaunchShape sh{1, 32 * run, 32};
+            float ms = 0;
+            rc = time_shape(ctx, fat, naik, copy, n, sh, in, out, flush, flush_bytes, &ms);
+            if (rc == HISQ_OK && ms < 0.98f * best_ms) {
+                best_ms = ms;
+                *best = sh;
+            }
+        }
     cudaStreamSynchronize(ctx->stream);
     cudaFree(in);
     cudaFree(out);
@@ -198,6 +209,16 @@ extern "C" int hisq_set_launch_shape(int prec, int recon, int nrhs, int rhs_per_
     int R = rhs_per_thread;
     if ((R != 1 && R != 2 && R != 4 && R != 8) || nrhs % R != 0 || (prec == HISQ_FP64 && R > 4))
         return set_error(HISQ_ERR_ARG, "rhs_per_thread %d is not available for nrhs %d", R, nrhs);
+    if (lanes_per_site == 32) {
+        // the tensor-core kernel as hisq_autotune reports it: 32 times the sites per run
+        if (prec < HISQ_FP16 || recon != 18 || R != 1 || nrhs < 2 || nrhs > 32 || (prec == HISQ_BF16 && nrhs % 2) ||
+            block_threads < 32 || block_threads > 1024 || block_threads % 32)
+            return set_error(HISQ_ERR_ARG, "32 lanes per site: 16-bit links, 18-real Naik records, 2..32 right-hand sides "
+                                           "(even for BF16), one per thread, block_threads 32 times 1..32 sites");
+        ctx->tuned[TuneKey{prec, recon, nrhs, 0}] = LaunchShape{R, block_threads, lanes_per_site};
+        ctx->tune_generation++;
+        return HISQ_OK;
+    }
     if (block_threads < 32 || block_threads > (lanes_per_site == 8 ? 512 : 256))
         return set_error(HISQ_ERR_ARG, "block_threads must be in 32..256 (32..512 staged)");
     if (lanes_per_site != 1 && !(lanes_per_site == 2 && recon == 18 && R <= 4) &&
