@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
 
     // ---- setup: x_hi = 0, x = 0, r = b, p = b and |b|^2 ----
     {
-        double acc[1] = {0.0};
+        DotSum<double> acc[1];
         if (row_ok) {
             for (int tile = blockIdx.x; (long)tile * ts < a.g.Vh; tile += gridDim.x) {
                 const int s = tile * ts + sl;
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
                 Cplx<rp> bp[3];
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    acc[0] += b[c].re * b[c].re + b[c].im * b[c].im;
+                    acc[0].add(b[c].re * b[c].re + b[c].im * b[c].im);
                     bq[c] = {(rq)b[c].re, (rq)b[c].im};
                     bp[c] = {(rp)b[c].re, (rp)b[c].im};
                 }
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
         // x += alpha p; r -= alpha A p with |r|^2 (for the next iteration's step); p = r + beta p,
         // except where an FP64 recomputation is due (there x_hi += x, x = 0, and p waits for the
         // true residual)
-        double rr_acc[1] = {0.0};
+        DotSum<rq> rr_acc[1];
         if (st.active[r] && row_ok) {
             const rq al = (rq)st.alpha[r][0];
             const rp be = (rp)st.beta[r][0];
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
                 rq part = 0;
 #pragma unroll
                 for (int c = 0; c < 3; c++) part += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
-                rr_acc[0] += (double)part;
+                rr_acc[0].add(part);
                 if (upd) {
                     Cplx<double> xh[3];
                     const Cplx<rq> zq[3] = {{0, 0}, {0, 0}, {0, 0}};
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
         clock_mark(clk, PH_AOP);
         // x += alpha p; r -= alpha A p; |r|^2
         {
-            double acc[1] = {0.0};
+            DotSum<rq> acc[1];
             if (st.active[r] && row_ok) {
                 const rq al = (rq)st.alpha[r][0];
                 for (int tile = blockIdx.x; (long)tile * ts < a.g.Vh; tile += gridDim.x) {
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
                         rv[c].im -= al * (rq)ap[c].im;
                         part += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
                     }
-                    acc[0] += (double)part;
+                    acc[0].add(part);
                     store_vec<Q>(VQ(x), s, r, x);
                     store_vec<Q>(VQ(r), s, r, rv);
                 }
