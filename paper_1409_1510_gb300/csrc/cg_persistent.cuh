@@ -169,13 +169,13 @@ struct DotSum<float> {
 };
 
 // Per-block column sums of the threads' dots into partials[blockIdx.x][col0 + *].  Thread
-// tid = site_row * t + gi holds dot[r] of column gi * R + r (ndots = t * R columns).  With t a
+// tid = site_row * t + gi holds dot[r] of column gi * cf + r * cs (by default gi * R + r; ndots columns).  With t a
 // power of two the lanes of one column meet in a shuffle tree and the warps' sums in one more
 // step; otherwise the dots go through red[rows][ndots] (red holds blockDim.x * R doubles).
 // With S lanes per thread position (tid = (site_row * t + gi) * S + part) the dots are in part 0.
 template <int R, int S = 1, typename T>
 __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, DotSum<T> (&dot)[R], int t, int gi,
-                                             int ndots, int col0 = 0) {
+                                             int ndots, int col0 = 0, int cf = R, int cs = 1) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int tS = t * S;
     const bool own = S == 1 || tid % S == 0;
@@ -187,7 +187,7 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, Dot
         if (lane < tS && own) {
 #pragma unroll
             for (int r = 0; r < R; r++)
-                if (gi * R + r < ndots) red[warp * ndots + gi * R + r] = dot[r].value();
+                if (gi * cf + r * cs < ndots) red[warp * ndots + gi * cf + r * cs] = dot[r].value();
         }
         __syncthreads();
         for (int j = warp; j < ndots; j += nwarps) {
@@ -204,7 +204,7 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, Dot
     if (row < rows && own) {
 #pragma unroll
         for (int r = 0; r < R; r++)
-            if (gi * R + r < ndots) red[row * ndots + gi * R + r] = dot[r].value();
+            if (gi * cf + r * cs < ndots) red[row * ndots + gi * cf + r * cs] = dot[r].value();
     }
     __syncthreads();
     for (int j = warp; j < ndots; j += nwarps) {
@@ -501,10 +501,10 @@ __device__ __forceinline__ void mma_phase(const PersArgs &a, const void *in, voi
 }
 
 // The FP64-accurate residual recomputation of a mixed-precision solve in double-single
-// arithmetic (ds_arith.cuh) over the block's share of the sites, one thread per site and DR
-// listed right-hand sides list[DR gi .. DR gi + DR) (nlist listed in all).  The solver uses
-// DR = 1: two right-hand sides per thread, which share each link load and give a thread two
-// independent accumulation chains, measured no faster at 64^3 x 16 with 16 right-hand sides.
+// arithmetic (ds_arith.cuh) over the block's share of the sites, one thread per site and DR listed
+// right-hand sides list[gi + r t] (nlist listed in all, t = ceil(nlist / DR) threads per site).  Kernels
+// with more than one right-hand side per thread take DR = 2: two share each link load and give a thread
+// twice the independent chains.
 // PF: prefetch the next link's operands (it made the persistent kernels spill, so they pass
 // false; the separate kernels of dslash_ds.cu prefetch).
 // EPI_PLAIN: out = D in (ds bundles).  EPI_RESID: r = b - m^2 x + D in with x, b FP64
@@ -522,8 +522,8 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
     int rr[DR];
 #pragma unroll
     for (int r = 0; r < DR; r++) {
-        act[r] = DR * gi + r < nlist;
-        rr[r] = act[r] ? list[DR * gi + r] : 0;
+        act[r] = gi + r * t < nlist;
+        rr[r] = act[r] ? list[gi + r * t] : 0;
     }
     DotSum<double> dot[DR];
     const int ts = tile_sites(g.Vh, spb);
@@ -579,7 +579,18 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
             }
         }
     }
-    if constexpr (EPI == EPI_RESID) publish_dots<DR, S>(a, red, dot, t, gi, nlist);
+    if constexpr (EPI == EPI_RESID) publish_dots<DR, S>(a, red, dot, t, gi, nlist, 0, 1, t);
+}
+
+// The same as a function of its own, so that its registers do not bear on the other phases' of a kernel
+// that has several right-hand sides per thread.  64^3 x 16, 16 FP16 right-hand sides, recomputations and
+// Dslash phases in ms: one right-hand side per thread, inlined 185 + 393; two, inlined 166 + 407; two in a
+// function of its own 172 + 385.  (One right-hand side, 32^3 x 16 FP16: inlined 2 % faster.)
+template <int EPI, int Q, int DR>
+__device__ __noinline__ void ds_phase_called(const PersArgs &a, const void *in, void *out, int parity,
+                                             const void *xvec, const void *bvec, void *out_lo, double *red,
+                                             const double *m2v, const int *list, int nlist) {
+    ds_phase<EPI, Q, DR, false>(a, in, out, parity, xvec, bvec, out_lo, red, m2v, list, nlist);
 }
 
 // x_hi of one site and right-hand side, written in double-single form for the recomputation

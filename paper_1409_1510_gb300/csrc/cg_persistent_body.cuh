@@ -37,8 +37,15 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
     dslash_phase<P, R, EPI, Q, PlainIn<P, true>, PlainIn<P, true>, DOTS2, S>(                                      \
         a, a.fat, a.naik, PlainIn<P, true>{VP(f)}, out, parity, st.active, PlainIn<P, true>{VP(p)}, nullptr, nullptr, \
         red, st.mass2)
-#define DS_PHASE(EPI, in, out, parity, x, b, lo) \
-    ds_phase<EPI, Q, 1, false, S>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n)
+#define DS_PHASE(EPI, in, out, parity, x, b, lo)                                                             \
+    do {                                                                                                     \
+        if constexpr (R == 1)                                                                                \
+            ds_phase<EPI, Q, 1, false, S>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);     \
+        else if (upd_n == 1)                                                                                 \
+            ds_phase_called<EPI, Q, 1>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);        \
+        else                                                                                                 \
+            ds_phase_called<EPI, Q, 2>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);        \
+    } while (0)
 
     // ---- setup: x_hi = 0, x = 0, r = b, p = b and |b|^2 ----
     {
