@@ -123,7 +123,9 @@ __device__ __forceinline__ bool grid_sync(const PersArgs &a) {
 // or with four lanes per site or the tensor-core phases (128 registers); the launch may use fewer (a
 // multiple of 32 dividing into the SM's resources).
 __host__ __device__ constexpr int pers_threads(int R, int S = 1) { return R == 1 && S == 1 ? 1024 : 512; }
-constexpr int PERS_SPLIT = -4;  // "R" of the kernel with four lanes per (site, right-hand side), R = 1
+// "R" = -S stands for the kernel with S lanes per (site, right-hand side), R = 1: four, or as many as a
+// precision's records have word-aligned groups of links (16-bit 4, FP32 8, FP64 16)
+__host__ __device__ constexpr int pers_most_lanes(int prec) { return prec == HISQ_FP64 ? 16 : prec == HISQ_FP32 ? 8 : 4; }
 constexpr int PERS_DEFAULT_THREADS = 512;  // measured best at 32^3 x 8 (one and 16 right-hand sides)
 
 // Sites per tile for a phase whose blocks cover spb sites at a time: when the grid covers the
@@ -319,7 +321,7 @@ __device__ __forceinline__ void sum_partials(const PersArgs &a, double *red, int
 // (ax from the loader `ax` at the output site); with DOTS2 also |out|^2, published as columns
 // 2n..3n-1 (columns n..2n-1 are left to the update phase's |r|^2).  EPI_RESID (FP64):
 // r = b - m^2 ax + D in, written to out_lo (iterated precision Q) with |r|^2 per block.  mask[r]
-// selects right-hand sides; m2v[r] is the m^2 of right-hand side r (shared memory).  S = 4: four lanes
+// selects right-hand sides; m2v[r] is the m^2 of right-hand side r (shared memory).  S > 1: S lanes
 // share a site and right-hand side (site_stencil's split), for lattices whose share per block leaves
 // most threads idle otherwise.
 template <int PP, int R, int EPI, int Q, class IN, class AX, bool DOTS2 = false, int S = 1>
@@ -510,7 +512,7 @@ __device__ __forceinline__ void mma_phase(const PersArgs &a, const void *in, voi
 // EPI_PLAIN: out = D in (ds bundles).  EPI_RESID: r = b - m^2 x + D in with x, b FP64
 // and an FP64 epilogue, written to out_lo in the iterated precision Q, with |r|^2 per block
 // published as column i of the list.
-// S = 4: four lanes per (site, right-hand side), four links each, on small lattices (see dslash_phase).
+// S > 1: S lanes per (site, right-hand side) on small lattices (see dslash_phase).
 template <int EPI, int Q, int DR, bool PF, int S = 1>
 __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void *out, int parity, const void *xvec,
                                          const void *bvec, void *out_lo, double *red, const double *m2v,
@@ -538,9 +540,10 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
                 ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
                                               rr, act, acc);
             } else {
-                static_assert(S == 4, "four lanes take four links each");
+                constexpr int PAIRS = 8 / S;  // (kind, direction) pairs per lane
+                static_assert(S == 4 || S == 8, "a lane takes both hops of its directions");
                 ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
-                                              rr, act, acc, 2 * part, valid ? 2 * part + 2 : 2 * part);
+                                              rr, act, acc, PAIRS * part, valid ? PAIRS * (part + 1) : PAIRS * part);
 #pragma unroll
                 for (int off = 1; off < S; off <<= 1)  // every lane of the warp takes part
 #pragma unroll

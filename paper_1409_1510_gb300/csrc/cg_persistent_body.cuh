@@ -339,12 +339,14 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
     }
 }
 
-// the instantiation for R right-hand sides per thread (FP64 stops at two: four would spill; PERS_SPLIT:
-// four lanes per site and right-hand side; MMA_GROUP: the tensor-core phases of 16-bit storage) and the
+// the instantiation for R right-hand sides per thread (FP64 stops at two: four would spill; R = -S:
+// S lanes per site and right-hand side; MMA_GROUP: the tensor-core phases of 16-bit storage) and the
 // CG form
 template <int P, bool CG1>
 const void *persistent_kernel_ptr(int R) {
-    if (R == PERS_SPLIT) return (const void *)cg_persistent_kernel<P, 1, CG1, 4>;
+    if (R == -4) return (const void *)cg_persistent_kernel<P, 1, CG1, 4>;
+    if constexpr (pers_most_lanes(P) > 4)
+        if (R == -pers_most_lanes(P)) return (const void *)cg_persistent_kernel<P, 1, CG1, pers_most_lanes(P)>;
     if constexpr (P == HISQ_FP16 || P == HISQ_BF16) {
         if (R == MMA_GROUP) return (const void *)cg_persistent_kernel<P, MMA_GROUP, CG1, 1>;
     }

@@ -446,8 +446,10 @@ __device__ __forceinline__ void site_stencil_pairs(const Geom &g, const LinkFiel
 // products of the site's links with the neighbouring input vectors (from the loader `vin`) of
 // the R right-hand sides r0.. that are active.  S = 1: all 16 links.  S = 2 (18-real Naik only):
 // the 8 fat (part 0) or the 8 Naik links (part 1).  S = 4 (18-real Naik only): part =
-// 2 kind + half, the four links of directions 2 half and 2 half + 1 of that kind.  Record slot 2 mu holds the forward link of
-// direction mu and slot 2 mu + 1 the backward one (already -U^dagger of the neighbour's link).
+// 2 kind + half, the four links of directions 2 half and 2 half + 1 of that kind; S = 8 and 16 halve and
+// quarter that where the records' word-aligned groups of links are as small (FP32 two, FP64 one).  Record
+// slot 2 mu holds the forward link of direction mu and slot 2 mu + 1 the backward one (already -U^dagger of
+// the neighbour's link).
 // 16-bit 18-real records carry one positive float scale per (parity, site) and field; it is
 // applied to the field's summed contribution (6 R products) instead of to the 18 reals of each
 // of its links: with both fields scaled, acc = s_N (s_X / s_N sum_X + sum_N).
@@ -469,21 +471,23 @@ __device__ __forceinline__ void site_stencil(const Geom &g, const LinkField &fat
     for (int r = 0; r < R; r++)
 #pragma unroll
         for (int c = 0; c < 3; c++) acc[r][c] = {0, 0};
-    if constexpr (S == 4) {
-        static_assert(NR == 18, "the four-lane split needs identical fat and Naik encodings");
-        const bool naik_kind = (part >> 1) != 0;
-        const int half = part & 1;
+    if constexpr (S >= 4) {
+        static_assert(NR == 18, "the split over four and more lanes needs identical fat and Naik encodings");
+        constexpr int H = S / 2;                    // lanes per kind
+        constexpr int GPL = FatC::GROUPS / H;       // groups per lane
+        static_assert(GPL >= 1 && GPL * H == FatC::GROUPS, "a lane takes whole groups of links");
+        const bool naik_kind = part >= H;
         const LinkField f = naik_kind ? naik_f : fat_f;
         const int hop = naik_kind ? 3 : 1;
-        constexpr int GPH = 4 / FatC::G;  // groups per half record (4 links)
 #pragma unroll
-        for (int gg = 0; gg < GPH; gg++) {
+        for (int gg = 0; gg < GPL; gg++) {
+            const int grp = (part % H) * GPL + gg;
             uint32_t u[FatC::WG * 4];
-            FatC::load_group(f, parity, g.Vh, s, half * GPH + gg, u);
+            FatC::load_group(f, parity, g.Vh, s, grp, u);
 #pragma unroll
             for (int l = 0; l < FatC::G; l++) {
-                const int j = gg * FatC::G + l;  // 0..3 within the half
-                const int nb = neighbour_rt(g, sc, s, 2 * half + (j >> 1), (j & 1) ? -hop : hop);
+                const int slot = grp * FatC::G + l;
+                const int nb = neighbour_rt(g, sc, s, slot >> 1, (slot & 1) ? -hop : hop);
                 Cplx<real> M[3][3];
                 FatC::decode(u, l, M);
                 Cplx<real> v[R][3];

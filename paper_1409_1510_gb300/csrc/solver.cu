@@ -886,11 +886,13 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     if ((S.prec == HISQ_FP32 || S.prec == HISQ_BF16) && R > 2) R = 2;
     while (S.n % R) R /= 2;
     // a lattice so small that with one block per SM every site and right-hand side of a block's share gets
-    // four lanes, each applying four links in place of 16 (beyond that the lanes would take turns).  At
-    // 8^3 x 4 a block has seven sites: one lane each left 9200 cycles of FP64 multiply-adds in one chain of
-    // instructions with 25 lanes idle; plain FP64 CG there 3.20 -> 1.43 ms
+    // four lanes, or as many as the precision allows (beyond that the lanes would take turns).  At 8^3 x 4 a
+    // block has seven sites: one lane each left 9200 cycles of FP64 multiply-adds in one chain of
+    // instructions with 25 lanes idle; plain FP64 CG there 3.20 ms, with four lanes 1.43, with 16 1.23
     const long share = (S.ctx->geom.Vh + S.ctx->num_sms - 1) / S.ctx->num_sms;
-    const bool split = S.ctx->params.persistent_threads == 0 && share * S.n * 4 <= PERS_DEFAULT_THREADS;
+    int lanes = pers_most_lanes(S.prec);
+    if (share * S.n * lanes > PERS_DEFAULT_THREADS) lanes = 4;
+    const bool split = S.ctx->params.persistent_threads == 0 && share * S.n * lanes <= PERS_DEFAULT_THREADS;
     if (split) R = 1;
     // the tensor-core phases where the tuner found that kernel the fastest for this bundle
     const bool mma = !split && sh.S == 32 && S.prec != HISQ_FP64 && S.n <= MMA_GROUP && mma_fields(S.fat, S.naik, S.n);
@@ -902,7 +904,7 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     const size_t smem = (size_t)(4 * threads * (mma ? 1 : R) + 64) * sizeof(double);  // four dot sets (single reduction)
     int per_sm = 0;
     const bool cg1 = S.ctx->params.single_reduction != 0;
-    const int kernel_R = split ? PERS_SPLIT : R;
+    const int kernel_R = split ? -lanes : R;
     if (persistent_occ(S.prec, kernel_R, cg1, threads, smem, &per_sm) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         return HISQ_OK;

@@ -275,3 +275,18 @@ def test_four_lanes_per_site_on_small_lattices(prec, dims, n):
             x, stats, iters, res = _solve(g, rhs, 0.1, inner_prec=prec, bundle=n, single_reduction=single)
             true = g.oracle.true_residual(np.stack(rhs), x, 0.1)
             assert np.all(true <= TOL * SLACK), (single, true)
+
+
+@pytest.mark.parametrize("prec,dims,n", [(0, (4, 4, 4, 4), 1), (0, (6, 4, 6, 4), 3), (0, (8, 8, 8, 4), 4),
+                                         (0, (8, 8, 8, 4), 5), (1, (4, 4, 4, 4), 1), (1, (8, 8, 8, 4), 9),
+                                         (1, (8, 8, 8, 4), 10)])
+def test_a_lane_per_link_group_on_small_lattices(prec, dims, n):
+    """The persistent solve with 16 (FP64) and 8 (FP32) lanes per site and right-hand side: sites and
+    right-hand sides whose lanes do not fill the warps, the last bundles taken on 152 SMs (seven sites x 4,
+    x 9) and the first that go back to four lanes; both CG forms, uneven norms."""
+    with gpu(dims, prec) as g:
+        rhs = [hi.gaussian_rhs(g.lat, 80 + k) * 10.0 ** (k % 4 - 2) for k in range(n)]
+        for single in (0, 1):
+            x, stats, iters, res = _solve(g, rhs, 0.1, inner_prec=prec, bundle=n, single_reduction=single)
+            true = g.oracle.true_residual(np.stack(rhs), x, 0.1)
+            assert np.all(true <= TOL * SLACK), (single, true)
