@@ -230,7 +230,8 @@ __global__ void __launch_bounds__(256, pc_layer_blocks(A, B, NR)) pc_layer_kerne
 // in lane i, which adds it to its FP64 sum.  A lane-by-lane reduction of every component of every
 // site, with lane 0 adding into FP64 sums in shared memory, was bound by those additions (75% of
 // the FP64 pipe, 5 ms for a 4 -> 4 layer): at 32^3 x 8 with 16 samples the loss and gradient took
-// 37.6 ms, with this kernel and the packed layers above 17.8 ms.
+// 37.6 ms, with this kernel and the packed layers above 17.8 ms; with one body of code for both hops
+// and link kinds 14.6 -> 13.9 ms (between the two the forward activations were kept instead of recomputed).
 struct PcGradArgs {
     PcLayerArgs L;       // in_same, in_opp: the layer input h; spb: sites per tile; out unused
     const float2 *G;     // gradient w.r.t. the layer output at the output parity
@@ -278,24 +279,41 @@ __device__ __forceinline__ void load_all(const float2 *f, int s, int k, int K, f
     for (int a0 = 0; a0 < C; a0 += PC_CHUNK<C>) load_chunk<C>(f, s, k, K, a0, h + a0);
 }
 
-// link 2 mu + DIR of a record (mu known at run time, the same for the whole warp)
-template <int NR, int DIR>
-__device__ __forceinline__ void load_direction(const LinkField &f, int parity, int Vh, int s, int mu,
-                                               Cplx<float> M[3][3]) {
+// link `slot` of a record (known at run time, the same for the whole warp)
+template <int NR>
+__device__ __forceinline__ void load_slot(const LinkField &f, int parity, int Vh, int s, int slot, Cplx<float> M[3][3]) {
     using C = LinkCodec<HISQ_FP32, NR>;
-    uint32_t u[C::WG * 4];
-    C::load_group(f, parity, Vh, s, 2 * mu / C::G, u);
     if constexpr (C::G == 2) {
-        C::decode(u, DIR, M);
+        // two 18-float links in nine words: the second starts in the middle of word 4
+        const bool odd = slot & 1;
+        const uint4 *w = f.words + ((size_t)parity * f.W + (slot >> 1) * 9 + (odd ? 4 : 0)) * Vh + s;
+        float u[20];
+#pragma unroll
+        for (int j = 0; j < 5; j++) {
+            const uint4 x = __ldg(w + (size_t)j * Vh);
+            u[4 * j] = __uint_as_float(x.x);
+            u[4 * j + 1] = __uint_as_float(x.y);
+            u[4 * j + 2] = __uint_as_float(x.z);
+            u[4 * j + 3] = __uint_as_float(x.w);
+        }
+#pragma unroll
+        for (int e = 0; e < 9; e++)
+            M[e / 3][e % 3] = {odd ? u[2 * e + 2] : u[2 * e], odd ? u[2 * e + 3] : u[2 * e + 1]};
     } else {
         static_assert(C::G == 4, "records of two or four links per group");
-        if (mu & 1) C::decode(u, 2 + DIR, M);
-        else C::decode(u, DIR, M);
+        uint32_t u[C::WG * 4];
+        C::load_group(f, parity, Vh, s, slot >> 2, u);
+        switch (slot & 3) {
+        case 0: C::decode(u, 0, M); break;
+        case 1: C::decode(u, 1, M); break;
+        case 2: C::decode(u, 2, M); break;
+        default: C::decode(u, 3, M);
+        }
     }
 }
 
-template <int A, int B, int NR, int DIR>
-__device__ __forceinline__ double grad_hop(const PcGradArgs &ga, const LinkField &f, int hop, int mu, int s0, int s1,
+template <int A, int B, int NR>
+__device__ __forceinline__ double grad_hop(const PcGradArgs &ga, const LinkField &f, int hop, int slot, int s0, int s1,
                                            int row, int rows, int k, int lane) {
     constexpr int N = PC_CHUNK<A>, NV = 2 * A * B;
     const PcLayerArgs &p = ga.L;
@@ -303,11 +321,12 @@ __device__ __forceinline__ double grad_hop(const PcGradArgs &ga, const LinkField
 #pragma unroll
     for (int i = 0; i < NV; i++) acc[i] = 0.f;
     if (row < rows) {
+#pragma unroll 1
         for (int s = s0 + row; s < s1; s += rows) {
             Cplx<float> M[3][3];
-            load_direction<NR, DIR>(f, p.parity, p.g.Vh, s, mu, M);
+            load_slot<NR>(f, p.parity, p.g.Vh, s, slot, M);
             const SiteCoord sc = decode_site(p.g, s, p.parity);
-            const int nb = neighbour_rt(p.g, sc, s, mu, DIR ? -hop : hop);
+            const int nb = neighbour_rt(p.g, sc, s, slot >> 1, (slot & 1) ? -hop : hop);
             float2 G[B][3];
             load_all<B>(ga.G, s, k, p.K, G);
 #pragma unroll
@@ -338,12 +357,21 @@ __global__ void __launch_bounds__(32 * PC_GRAD_WARPS, 2) pc_grad_kernel(PcGradAr
     for (int tile = blockIdx.x; (long)tile * p.spb < p.g.Vh; tile += gridDim.x, turn++) {
         const int s0 = tile * p.spb, s1 = min(s0 + p.spb, p.g.Vh);
         if (p.in_opp) {
-            if (naik_kind) {
-                fwd += grad_hop<A, B, NR, 0>(ga, p.naik, 3, mu, s0, s1, row, rows, k, lane);
-                bwd += grad_hop<A, B, NR, 1>(ga, p.naik, 3, mu, s0, s1, row, rows, k, lane);
-            } else {
-                fwd += grad_hop<A, B, 18, 0>(ga, p.fat, 1, mu, s0, s1, row, rows, k, lane);
-                bwd += grad_hop<A, B, 18, 1>(ga, p.fat, 1, mu, s0, s1, row, rows, k, lane);
+            // one body of code for every warp and both hops where the two encodings agree: with a body per
+            // hop and kind, the warps at different places of four bodies, waiting for instructions was the
+            // largest stall (3.3 warps per instruction issued in a 4 -> 4 layer; now 0.04)
+#pragma unroll 1
+            for (int dir = 0; dir < 2; dir++) {
+                double sum;
+                if constexpr (NR == 18) {
+                    sum = grad_hop<A, B, 18>(ga, naik_kind ? p.naik : p.fat, naik_kind ? 3 : 1, 2 * mu + dir, s0, s1, row,
+                                             rows, k, lane);
+                } else {
+                    if (naik_kind) sum = grad_hop<A, B, NR>(ga, p.naik, 3, 2 * mu + dir, s0, s1, row, rows, k, lane);
+                    else sum = grad_hop<A, B, 18>(ga, p.fat, 1, 2 * mu + dir, s0, s1, row, rows, k, lane);
+                }
+                if (dir) bwd += sum;
+                else fwd += sum;
             }
         }
         if (p.in_same && (turn & (PC_GRAD_WARPS - 1)) == warp) {
