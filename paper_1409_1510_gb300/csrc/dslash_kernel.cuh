@@ -64,10 +64,10 @@ __device__ __forceinline__ VecView<P> view(const void *base, int Vh, int n) {
 // last-block-done finish: the block that takes the last ticket sums the partials of all blocks
 // in a fixed order, writes dot_out and runs the hook for a bundle of hook_n right-hand sides.
 // No block ever waits for another.  All threads of the block call it; blockDim.x is a multiple
-// of 32; ndots may be 0 (hook only); red holds at least blockDim.x + 64 doubles, and 2 * ndots
-// when ndots > 64.  Block column sums run one warp per column (lanes stride over the rows and
-// finish with a shuffle tree); the last block gives each thread one column and a stride of the
-// blocks' partials, so each stage needs a single barrier.
+// of 32; ndots is at most 64 and may be 0 (hook only); red holds at least blockDim.x + 64 doubles.
+// Block column sums run one warp per column (lanes stride over the rows and finish with a shuffle
+// tree); the last block gives each thread one column and a stride of the blocks' partials, so each
+// stage needs a single barrier.
 __device__ __forceinline__ void block_reduce_finish(double *red, int rows, int ndots, int hook_n, const RedArgs &ra) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     __shared__ int is_last;
@@ -93,49 +93,33 @@ __device__ __forceinline__ void block_reduce_finish(double *red, int rows, int n
     __syncthreads();
     if (ndots > 0) {
         const int nb = gridDim.x;
-        if (ndots <= 64) {
-            // thread (k, j), j < np2 (ndots padded to a power of two), sums column j over blocks
-            // k, k + per, ...; lanes of one column are np2 apart in a warp and meet in a shuffle
-            // tree, then at most 8 warp sums per column are added in a fixed order
-            int np2 = 1;
-            while (np2 < ndots) np2 *= 2;
-            const int per = blockDim.x / np2;
-            const int j = tid % np2, k = tid / np2;
-            double s = 0.0;
-            if (j < ndots && k < per) {
+        // thread (k, j), j < np2 (ndots padded to a power of two), sums column j over blocks
+        // k, k + per, ...; lanes of one column are np2 apart in a warp and meet in a shuffle
+        // tree, then at most 8 warp sums per column are added in a fixed order
+        int np2 = 1;
+        while (np2 < ndots) np2 *= 2;
+        const int per = blockDim.x / np2;
+        const int j = tid % np2, k = tid / np2;
+        double s = 0.0;
+        if (j < ndots && k < per) {
 #pragma unroll 4
-                for (int b = k; b < nb; b += per) s += __ldcg(ra.partials + (size_t)b * ndots + j);
-            }
-            for (int off = 16; off >= np2; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            const int groups = np2 < 32 ? nwarps : per;           // partial sums per column
-            if (np2 < 32) {
-                if (lane < np2) red[warp * np2 + lane] = s;
-            } else {
-                red[tid] = s;
-            }
-            __syncthreads();
-            if (tid < ndots) {
-                double t = 0.0;
-                for (int q = 0; q < groups; q++) t += red[q * np2 + tid];
-                red[blockDim.x + tid] = t;
-            }
-            __syncthreads();
-            if (tid < ndots) red[tid] = red[blockDim.x + tid];
-        } else {
-            // many columns (network weight gradients): one thread per column
-            // (four sums in flight: an FP64 add is a 64-cycle dependent operation)
-            for (int j = tid; j < ndots; j += blockDim.x) {
-                double t[4] = {0.0, 0.0, 0.0, 0.0};
-                int b = 0;
-                for (; b + 4 <= nb; b += 4)
-#pragma unroll
-                    for (int u = 0; u < 4; u++) t[u] += __ldcg(ra.partials + (size_t)(b + u) * ndots + j);
-                for (; b < nb; b++) t[0] += __ldcg(ra.partials + (size_t)b * ndots + j);
-                red[ndots + j] = (t[0] + t[1]) + (t[2] + t[3]);
-            }
-            __syncthreads();
-            for (int j = tid; j < ndots; j += blockDim.x) red[j] = red[ndots + j];
+            for (int b = k; b < nb; b += per) s += __ldcg(ra.partials + (size_t)b * ndots + j);
         }
+        for (int off = 16; off >= np2; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        const int groups = np2 < 32 ? nwarps : per;           // partial sums per column
+        if (np2 < 32) {
+            if (lane < np2) red[warp * np2 + lane] = s;
+        } else {
+            red[tid] = s;
+        }
+        __syncthreads();
+        if (tid < ndots) {
+            double t = 0.0;
+            for (int q = 0; q < groups; q++) t += red[q * np2 + tid];
+            red[blockDim.x + tid] = t;
+        }
+        __syncthreads();
+        if (tid < ndots) red[tid] = red[blockDim.x + tid];
         __syncthreads();
         if (ra.dot_out)
             for (int j = tid; j < ndots; j += blockDim.x) ra.dot_out[j] = red[j];

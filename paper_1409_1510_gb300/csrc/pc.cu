@@ -137,7 +137,9 @@ static int ensure_work(hisq_ctx *ctx, hisq_pc *pc, int K) {
     free_work(w);
     size_t Vh = ctx->geom.Vh;
     size_t f4 = Vh * 3 * K * 4 * sizeof(float2), f1 = Vh * 3 * K * sizeof(float2);
-    size_t pcap = (size_t)ctx->num_sms * 8 * PC_PATHS * 16 * 2;
+    size_t pcap = (size_t)ctx->num_sms * 8 * PC_PATHS * 16 * 2;  // eight blocks of 256 threads fill an SM
+    // the finished blocks or groups, and the blocks of each group of a gradient kernel
+    const size_t counters = sizeof(unsigned int) * (1 + (ctx->num_sms * 8 + PC_GRAD_GROUP - 1) / PC_GRAD_GROUP);
     bool ok = true;
     for (int p = 0; p < 2; p++)
         ok = ok && cudaMalloc(&w.h1[p], f4) == cudaSuccess && cudaMalloc(&w.h2[p], f4) == cudaSuccess &&
@@ -153,13 +155,13 @@ static int ensure_work(hisq_ctx *ctx, hisq_pc *pc, int K) {
          cudaMalloc(&w.err2, sizeof(double) * HISQ_MAX_BUNDLE) == cudaSuccess &&
          cudaMalloc(&w.grad, sizeof(double) * 2 * HISQ_PC_WEIGHTS) == cudaSuccess &&
          cudaMalloc(&w.partials, sizeof(double) * pcap) == cudaSuccess &&
-         cudaMalloc(&w.counter, sizeof(unsigned int) * 4) == cudaSuccess;
+         cudaMalloc(&w.counter, counters) == cudaSuccess;
     if (!ok) {
         free_work(w);
         return set_error(HISQ_ERR_NOMEM, "preconditioner workspace allocation failed");
     }
     w.partials_cap = pcap;
-    cudaMemset(w.counter, 0, sizeof(unsigned int) * 4);
+    cudaMemset(w.counter, 0, counters);
     w.K = K;
     return HISQ_OK;
 }
@@ -233,14 +235,14 @@ static int run_layer(hisq_ctx *ctx, const hisq_links *naik, const PcLayerArgs &p
 template <int A, int B>
 static int run_grad(hisq_ctx *ctx, const hisq_links *naik, PcWork &w, PcGradArgs ga, cudaStream_t st) {
     constexpr int ND = PC_PATHS * A * B * 2;
-    const size_t smem = std::max(2 * ND, 32 * PC_GRAD_WARPS + 64) * sizeof(double);
+    const size_t smem = ND * sizeof(double);
     // a tile gives every lane eight (site, sample) pairs per path, fewer where the lattice would not
     // fill the GPU
     const int rows = 32 / ga.L.K;
     ga.L.spb = rows * (int)std::max(1L, std::min(8L, (long)ctx->geom.Vh / ((long)rows * ctx->num_sms * 2)));
     auto launch = [&](auto k) -> int {
         int grid = grid_of(ctx, k, smem, ga.L.spb);
-        if ((size_t)grid * ND > w.partials_cap) grid = (int)(w.partials_cap / ND);
+        grid = std::min(grid, ctx->num_sms * 8);  // partials and counters
         k<<<grid, 32 * PC_GRAD_WARPS, smem, st>>>(ga);
         return HISQ_OK;
     };

@@ -231,14 +231,17 @@ __global__ void __launch_bounds__(256, pc_layer_blocks(A, B, NR)) pc_layer_kerne
 // site, with lane 0 adding into FP64 sums in shared memory, was bound by those additions (75% of
 // the FP64 pipe, 5 ms for a 4 -> 4 layer): at 32^3 x 8 with 16 samples the loss and gradient took
 // 37.6 ms, with this kernel and the packed layers above 17.8 ms; with one body of code for both hops
-// and link kinds 14.6 -> 13.9 ms (between the two the forward activations were kept instead of recomputed).
+// and link kinds 14.6 -> 13.9 ms (between the two the forward activations were kept instead of
+// recomputed); with the blocks' sums added in groups (grad_finish) and three blocks per SM for the layers
+// of four weights 13.9 -> 12.95 ms.
 struct PcGradArgs {
     PcLayerArgs L;       // in_same, in_opp: the layer input h; spb: sites per tile; out unused
     const float2 *G;     // gradient w.r.t. the layer output at the output parity
     RedArgs red;
 };
 
-constexpr int PC_GRAD_WARPS = 8;  // four directions of two link kinds
+constexpr int PC_GRAD_WARPS = 8;   // four directions of two link kinds
+constexpr int PC_GRAD_GROUP = 16;  // blocks whose partials are added first
 
 // v[0 .. N): in lane l afterwards v[0] = the warp's sum of component l % N (N a power of two <= 32)
 template <int N>
@@ -342,8 +345,58 @@ __device__ __forceinline__ double grad_hop(const PcGradArgs &ga, const LinkField
     return (double)acc[0];
 }
 
+// s[j] = sum over rows of row[r * stride + j] (four sums in flight: an FP64 add is a 64-cycle dependent
+// operation), for the thread's columns j
+template <int ND, typename F>
+__device__ __forceinline__ void sum_rows(const double *row, size_t stride, int rows, F &&put) {
+    for (int j = threadIdx.x; j < ND; j += blockDim.x) {
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        int b = 0;
+        for (; b + 4 <= rows; b += 4)
+#pragma unroll
+            for (int u = 0; u < 4; u++) t[u] += __ldcg(row + (size_t)(b + u) * stride + j);
+        for (; b < rows; b++) t[0] += __ldcg(row + (size_t)b * stride + j);
+        put(j, (t[0] + t[1]) + (t[2] + t[3]));
+    }
+}
+
+// The sums of the blocks' ND columns (red, shared memory) into dot_out, in a fixed order and with no block
+// waiting for another: the block that finishes last of its group of 16 adds the group's partials, the
+// group that finishes last adds the groups' sums.  One last block adding the partials of all 304 was a
+// sixth of the time of a 4 -> 4 layer's kernel, and a fence per column more before it.
+// ra.counter: one counter for the groups and then one per group, zero before and after.
+template <int ND>
+__device__ __forceinline__ void grad_finish(const double *red, const RedArgs &ra) {
+    __shared__ int last;
+    const int nb = gridDim.x, g = blockIdx.x / PC_GRAD_GROUP, groups = (nb + PC_GRAD_GROUP - 1) / PC_GRAD_GROUP;
+    const int size = min(PC_GRAD_GROUP, nb - g * PC_GRAD_GROUP);
+    double *mine = ra.partials + (size_t)g * PC_GRAD_GROUP * ND;
+    __syncthreads();
+    for (int j = threadIdx.x; j < ND; j += blockDim.x) ra.partials[(size_t)blockIdx.x * ND + j] = red[j];
+    __threadfence();  // publish before the ticket is taken
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ra.counter + 1 + g, 1u) == size - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sum_rows<ND>(mine, ND, size, [&](int j, double s) { mine[j] = s; });
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ra.counter[1 + g] = 0u;
+        last = atomicAdd(ra.counter, 1u) == groups - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    sum_rows<ND>(ra.partials, (size_t)PC_GRAD_GROUP * ND, groups, [&](int j, double s) { ra.dot_out[j] = s; });
+    if (threadIdx.x == 0) ra.counter[0] = 0u;
+}
+
+// three blocks per SM where the sums of a path are eight (80 registers): the loss and gradient above 1.2 %
+// faster than with two; four per SM (64 registers) spill and gain nothing more.  4 -> 4 layers need the 128.
 template <int A, int B, int NR>
-__global__ void __launch_bounds__(32 * PC_GRAD_WARPS, 2) pc_grad_kernel(PcGradArgs ga) {
+__global__ void __launch_bounds__(32 * PC_GRAD_WARPS, A * B < 16 ? 3 : 2) pc_grad_kernel(PcGradArgs ga) {
     constexpr int N = PC_CHUNK<A>, NV = 2 * A * B, ND = PC_PATHS * NV;  // doubles per partial
     extern __shared__ double red[];
     __shared__ double same[PC_GRAD_WARPS][NV];
@@ -406,7 +459,7 @@ __global__ void __launch_bounds__(32 * PC_GRAD_WARPS, 2) pc_grad_kernel(PcGradAr
         for (int w = 0; w < PC_GRAD_WARPS; w++) s += same[w][threadIdx.x];
         red[threadIdx.x] = s;
     }
-    block_reduce_finish(red, 1, ND, 0, ga.red);
+    grad_finish<ND>(red, ga.red);
 }
 
 }  // namespace hisq

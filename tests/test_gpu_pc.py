@@ -75,6 +75,26 @@ def test_loss_and_gradient_parity(K):
         assert np.linalg.norm(got - want_grad) / np.linalg.norm(want_grad) <= 1e-4
 
 
+@pytest.mark.parametrize("dims,K,recon", [((4, 4, 4, 4), 1, 18), ((4, 4, 4, 4), 16, 13), ((4, 4, 4, 6), 7, 9),
+                                          ((4, 4, 6, 6), 16, 18), ((6, 6, 6, 6), 16, 18), ((6, 6, 6, 6), 16, 13)])
+def test_gradient_sums_over_few_and_many_blocks(dims, K, recon):
+    """The gradient kernel's two-stage sums: one incomplete group of blocks, whole groups, a last group of
+    a few blocks; every Naik encoding (nine reals rebuild a link to 5e-5, three layers apply one each)."""
+    with gpu(dims, 1, recon) as g:
+        W = _weights(5, 0.2)
+        pc = g.hisq.hisq_pc_create(_as_real(W))
+        g.hisq.hisq_pc_set_form(pc, g.hisq.HISQ_PC_HERMITIAN_PART)
+        r = np.stack([hi.gaussian_rhs(g.lat, 110 + k) for k in range(K)])
+        e = np.stack([hi.gaussian_rhs(g.lat, 130 + k) for k in range(K)])
+        want_loss, want_grad = g.oracle.pc_loss_grad(W, r, e, 0.2)
+        for _ in range(2):  # the counters are left as they were found
+            grad = np.zeros(2 * NW)
+            loss = g.hisq.hisq_pc_loss_grad(pc, g.fat, g.naik, 0.2, g.pack(r, 1), g.pack(e, 1), K, grad)
+            assert abs(loss - want_loss) / want_loss <= (1e-5 if recon != 9 else 3e-4)
+            got = grad.view(np.complex128)
+            assert np.linalg.norm(got - want_grad) / np.linalg.norm(want_grad) <= (1e-4 if recon != 9 else 3e-4)
+
+
 def test_adam_step_matches_oracle():
     with gpu((4, 4, 4, 4), 1) as g:
         W = _weights(3)
