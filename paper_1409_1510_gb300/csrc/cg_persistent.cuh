@@ -549,10 +549,7 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
 #pragma unroll
                     for (int r = 0; r < DR; r++)
 #pragma unroll
-                        for (int c = 0; c < 3; c++) {
-                            acc[r][c].re = ds_add_lane(acc[r][c].re, off);
-                            acc[r][c].im = ds_add_lane(acc[r][c].im, off);
-                        }
+                        for (int c = 0; c < 3; c++) acc[r][c] = ds_add_lane(acc[r][c], off);
                 if (!valid || part != 0) continue;
             }
 #pragma unroll
@@ -571,8 +568,8 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
                     for (int c = 0; c < 3; c++) {
                         const long idx = ((long)s * 3 + c) * n + rr[r];
                         const double2 x = __ldcg(vx + idx), b = __ldcg(vb + idx);
-                        const double wr = b.x - m2 * x.x + ds_value(acc[r][c].re);
-                        const double wi = b.y - m2 * x.y + ds_value(acc[r][c].im);
+                        const double wr = b.x - m2 * x.x + ds_value(acc[r][c].re());
+                        const double wi = b.y - m2 * x.y + ds_value(acc[r][c].im());
                         d += wr * wr + wi * wi;
                         lo3[c] = {(typename Prec<Q>::real)wr, (typename Prec<Q>::real)wi};
                     }
@@ -587,8 +584,9 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
 
 // The same as a function of its own, so that its registers do not bear on the other phases' of a kernel
 // that has several right-hand sides per thread.  64^3 x 16, 16 FP16 right-hand sides, recomputations and
-// Dslash phases in ms: one right-hand side per thread, inlined 185 + 393; two, inlined 166 + 407; two in a
-// function of its own 172 + 385.  (One right-hand side, 32^3 x 16 FP16: inlined 2 % faster.)
+// Dslash phases in ms (then in scalar double-single arithmetic): one right-hand side per thread, inlined
+// 185 + 393; two, inlined 166 + 407; two in a function of its own 172 + 385.  (Solves of one right-hand
+// side, 32^3 x 8 FP16: inlined 3 % faster.)
 template <int EPI, int Q, int DR>
 __device__ __noinline__ void ds_phase_called(const PersArgs &a, const void *in, void *out, int parity,
                                              const void *xvec, const void *bvec, void *out_lo, double *red,

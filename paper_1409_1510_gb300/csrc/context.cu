@@ -99,7 +99,7 @@ __device__ inline void gathered_link(const Geom &g, const double *U, const int c
 
 template <int P>
 __host__ __device__ constexpr int stored_real_bytes() {
-    if constexpr (P == HISQ_DS) return 8;  // the (hi, lo) float pair
+    if constexpr (P == HISQ_DS) return 8;  // a float pair; a complex number's word is (re_hi, im_hi, re_lo, im_lo)
     else return Prec<P>::bytes;
 }
 
@@ -112,8 +112,9 @@ __device__ inline void put_real(uint4 *words, int Vh, int W, int parity, int s, 
     if constexpr (P == HISQ_FP64) *reinterpret_cast<double *>(base) = val;
     else if constexpr (P == HISQ_DS) {
         const float hi = __double2float_rn(val);
-        reinterpret_cast<float *>(base)[0] = hi;
-        reinterpret_cast<float *>(base)[1] = __double2float_rn(val - (double)hi);
+        float *word = reinterpret_cast<float *>(base - b);  // (re_hi, im_hi, re_lo, im_lo)
+        word[e & 1] = hi;
+        word[2 + (e & 1)] = __double2float_rn(val - (double)hi);
     }
     else if constexpr (P == HISQ_FP32) *reinterpret_cast<float *>(base) = (float)val;
     else if constexpr (P == HISQ_FP16) *reinterpret_cast<__half *>(base) = __double2half(val);

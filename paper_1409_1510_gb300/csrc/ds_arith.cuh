@@ -14,11 +14,11 @@
 // costs here run about six times faster than one FP64 fused multiply-add.
 //
 // The error-free steps use the rounding intrinsics (__fmul_rn, __fadd_rn, __fsub_rn, __fmaf_rn),
-// which the compiler neither contracts into fused operations nor reorders.
+// which the compiler neither contracts into fused operations nor reorders, or their packed forms below.
 //
-// Storage: a ds link record has the FP64 record's layout (8 bytes per real) with every double
-// replaced by its (hi, lo) float pair; a ds colour vector bundle has the FP64 bundle's layout
-// with every complex number (re, im) stored as the float4 (re_hi, re_lo, im_hi, im_lo).
+// Storage: a ds link record has the FP64 record's layout (16 bytes per complex number) with every
+// complex number as the float4 (re_hi, im_hi, re_lo, im_lo); a ds colour vector bundle has the FP64
+// bundle's layout with every complex number (re, im) stored as the float4 (re_hi, re_lo, im_hi, im_lo).
 #pragma once
 #include "hisq_internal.cuh"
 
@@ -28,20 +28,55 @@ struct dsacc {
     float hi, lo;
 };
 
-// s += a b for ds numbers a = (a_hi, a_lo), b = (b_hi, b_lo).  With p = fl(a_hi b_hi) and t = fl(s.hi + p),
-// two-sum gives z = fl(t - s.hi) and the error (s.hi - (t - z)) + (p - z); p - z is exact, so one fused
-// multiply-add, a_hi b_hi - z, is that second part together with the product's own error a_hi b_hi - p:
-// ten operations in place of twelve (residual recomputations of the 64^3 x 16 solve 206 -> 198 ms), the
-// same error.
-__device__ __forceinline__ void ds_mac(dsacc &s, float a_hi, float a_lo, float b_hi, float b_lo) {
-    const float p = __fmul_rn(a_hi, b_hi);
-    const float t = __fadd_rn(s.hi, p);
-    const float z = __fsub_rn(t, s.hi);
-    const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, z)), __fmaf_rn(a_hi, b_hi, -z));
-    float lo = __fmaf_rn(a_hi, b_lo, s.lo);
-    lo = __fmaf_rn(a_lo, b_hi, lo);
+// A complex ds accumulator, real and imaginary part in the two halves of a packed pair.
+struct dscplx {
+    float2 hi, lo;
+    __device__ __forceinline__ dsacc re() const { return {hi.x, lo.x}; }
+    __device__ __forceinline__ dsacc im() const { return {hi.y, lo.y}; }
+};
+
+// Packed operations on (re, im) with one rounding each, written in PTX.  A packed product followed by a
+// packed sum is fused into one multiply-add by the assembler in spite of the .rn, which two-sum does not
+// survive (errors of 1e-8 in place of 1e-13); a product plus zero is not.
+union ds_pair {
+    float2 f;
+    unsigned long long u;
+    __device__ __forceinline__ ds_pair(float2 x) : f(x) {}
+    __device__ __forceinline__ ds_pair() {}
+};
+__device__ __forceinline__ float2 ds_mul2(ds_pair a, ds_pair b) {
+    ds_pair d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.u) : "l"(a.u), "l"(b.u), "l"(0ull));
+    return d.f;
+}
+__device__ __forceinline__ float2 ds_add2(ds_pair a, ds_pair b) {
+    ds_pair d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.u) : "l"(a.u), "l"(b.u));
+    return d.f;
+}
+__device__ __forceinline__ float2 ds_fma2(ds_pair a, ds_pair b, ds_pair c) {
+    ds_pair d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.u) : "l"(a.u), "l"(b.u), "l"(c.u));
+    return d.f;
+}
+__device__ __forceinline__ float2 ds_sub2(float2 a, float2 b) { return ds_fma2(b, make_float2(-1.f, -1.f), a); }
+
+// s += a b, both halves, for ds numbers a = (a_hi, a_lo), b = (b_hi, b_lo).  With p = fl(a_hi b_hi) and
+// t = fl(s.hi + p), two-sum gives z = fl(t - s.hi) and the error (s.hi - (t - z)) + (p - z); p - z is exact,
+// so one fused multiply-add, a_hi b_hi - z, is that second part together with the product's own error
+// a_hi b_hi - p: ten operations in place of twelve, the same error.  (nz = s.hi - t = -z exactly.)
+// Packed against scalar: half the instructions and twice the independent work of each, on kernels that keep
+// the FP32 pipe 40 % busy (latency, 16 and fewer warps per SM): residual of 4 right-hand sides at 32^3 x 8
+// 403 -> 347 us, of one 160 -> 142, recomputations of the 64^3 x 16 solve of 16 171 -> 157 ms.
+__device__ __forceinline__ void ds_mac(dscplx &s, float2 a_hi, float2 a_lo, float2 b_hi, float2 b_lo) {
+    const float2 p = ds_mul2(a_hi, b_hi);
+    const float2 t = ds_add2(s.hi, p);
+    const float2 nz = ds_sub2(s.hi, t);
+    const float2 err = ds_add2(ds_sub2(s.hi, ds_add2(t, nz)), ds_fma2(a_hi, b_hi, nz));
+    float2 lo = ds_fma2(a_hi, b_lo, s.lo);
+    lo = ds_fma2(a_lo, b_hi, lo);
     s.hi = t;
-    s.lo = __fadd_rn(lo, err);
+    s.lo = ds_add2(lo, err);
 }
 
 // the pair (hi, lo) with hi = fl(hi + lo): the accumulator in the storage form
@@ -60,6 +95,10 @@ __device__ __forceinline__ dsacc ds_add_lane(dsacc s, int off) {
     const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, z)), __fsub_rn(hi, z));
     return {t, __fadd_rn(__fadd_rn(s.lo, lo), err)};
 }
+__device__ __forceinline__ dscplx ds_add_lane(const dscplx &s, int off) {
+    const dsacc re = ds_add_lane(s.re(), off), im = ds_add_lane(s.im(), off);
+    return {make_float2(re.hi, im.hi), make_float2(re.lo, im.lo)};
+}
 
 __device__ __forceinline__ double ds_value(dsacc s) { return (double)s.hi + (double)s.lo; }
 
@@ -68,12 +107,8 @@ __device__ __forceinline__ void ds_split(double x, float &hi, float &lo) {
     lo = __double2float_rn(x - (double)hi);
 }
 
-// A complex ds accumulator and the ds colour-vector bundle (float4 per complex number at
-// (s * 3 + c) * n + r, like the FP64 bundle's double2).
-struct dscplx {
-    dsacc re, im;
-};
-
+// The ds colour-vector bundle: float4 per complex number at (s * 3 + c) * n + r, like the FP64 bundle's
+// double2.
 template <bool COHERENT>
 __device__ __forceinline__ float4 ds_load(const float4 *v, long idx) {
     if constexpr (COHERENT) return __ldcg(v + idx);
@@ -83,29 +118,26 @@ __device__ __forceinline__ float4 ds_load(const float4 *v, long idx) {
 __device__ __forceinline__ void ds_store3(float4 *v, int n, long s, int r, const dscplx w[3]) {
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-        const dsacc re = ds_normalize(w[c].re), im = ds_normalize(w[c].im);
+        const dsacc re = ds_normalize(w[c].re()), im = ds_normalize(w[c].im());
         v[(s * 3 + c) * n + r] = make_float4(re.hi, re.lo, im.hi, im.lo);
     }
 }
 
 // acc[a] += M_ab v_b for the three rows a of column b of one ds link: m[a] = the 16-byte word of
-// entry (a, b), i.e. the floats (re_hi, re_lo, im_hi, im_lo), and one ds colour component v_b.
-// The six accumulators (three rows, real and imaginary part) are independent chains, so a thread
-// keeps six two-sum sequences in flight instead of two.
+// entry (a, b), i.e. the floats (re_hi, im_hi, re_lo, im_lo), and one ds colour component v_b.
+// (mr, mi) vr first, then (-mi, mr) vi: both parts of a complex number in one packed operation.
+// The six accumulators (three rows, real and imaginary part) are independent chains.
 __device__ __forceinline__ void ds_column_acc(const uint4 m[3], const float4 vb, dscplx acc[3]) {
+    const float2 vr_hi = make_float2(vb.x, vb.x), vr_lo = make_float2(vb.y, vb.y);
+    const float2 vi_hi = make_float2(vb.z, vb.z), vi_lo = make_float2(vb.w, vb.w);
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const float mr_hi = __uint_as_float(m[a].x), mr_lo = __uint_as_float(m[a].y);
-        // (mr + i mi)(vr + i vi): the mr products first, the mi products below
-        ds_mac(acc[a].re, mr_hi, mr_lo, vb.x, vb.y);
-        ds_mac(acc[a].im, mr_hi, mr_lo, vb.z, vb.w);
-    }
+    for (int a = 0; a < 3; a++)
+        ds_mac(acc[a], make_float2(__uint_as_float(m[a].x), __uint_as_float(m[a].y)),
+               make_float2(__uint_as_float(m[a].z), __uint_as_float(m[a].w)), vr_hi, vr_lo);
 #pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const float mi_hi = __uint_as_float(m[a].z), mi_lo = __uint_as_float(m[a].w);
-        ds_mac(acc[a].re, -mi_hi, -mi_lo, vb.z, vb.w);
-        ds_mac(acc[a].im, mi_hi, mi_lo, vb.x, vb.y);
-    }
+    for (int a = 0; a < 3; a++)
+        ds_mac(acc[a], make_float2(-__uint_as_float(m[a].y), __uint_as_float(m[a].x)),
+               make_float2(-__uint_as_float(m[a].w), __uint_as_float(m[a].z)), vi_hi, vi_lo);
 }
 
 // the 9 words of one link of a ds record and the neighbour vectors it multiplies
@@ -153,7 +185,7 @@ __device__ __forceinline__ void ds_site_stencil(const Geom &g, const LinkField &
 #pragma unroll
     for (int r = 0; r < R; r++)
 #pragma unroll
-        for (int c = 0; c < 3; c++) acc[r][c] = {{0.f, 0.f}, {0.f, 0.f}};
+        for (int c = 0; c < 3; c++) acc[r][c] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     // first word of the forward link of pair k; the backward one is nine planes on
     auto words = [&](int k) {
         const LinkField &f = k >= 4 ? naik : fat;

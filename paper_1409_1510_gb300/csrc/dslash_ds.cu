@@ -91,8 +91,8 @@ __global__ void __launch_bounds__(256, R == 1 ? 2 : 1) dslash_ds_kernel(KArgs a)
                     const long idx = a.canon ? ((long)(r0 + r) * g.Vh + s) * 3 + c : ((long)s * 3 + c) * a.n + r0 + r;
                     const long bidx = a.b_one ? (long)s * 3 + c : idx;
                     const double2 x = __ldg(vx + idx), b = __ldg(vb + bidx);
-                    w[c].x = b.x - m2 * x.x + ds_value(acc[r][c].re);
-                    w[c].y = b.y - m2 * x.y + ds_value(acc[r][c].im);
+                    w[c].x = b.x - m2 * x.x + ds_value(acc[r][c].re());
+                    w[c].y = b.y - m2 * x.y + ds_value(acc[r][c].im());
                     d += w[c].x * w[c].x + w[c].y * w[c].y;
                 }
                 dot[r] += d;
@@ -199,7 +199,7 @@ extern "C" int hisq_residual(const hisq_links *fat, const hisq_links *naik, doub
     const size_t total = staging + (ds ? 2 : 4) * vb + pbytes + 256;
     // scratch: staging, then x (ds) and t, or b, x, t, r (FP64); partials; counter.  Kept in the context up
     // to HISQ_RESID_KEEP.  4 right-hand sides at 32^3 x 8: 707 us with an allocation per call and staging
-    // copies, packs and unpacks around the two Dslash kernels, 416 us now
+    // copies, packs and unpacks around the two Dslash kernels, 416 without them
     char *buf = nullptr, *owned = nullptr;
     if (total <= HISQ_RESID_KEEP) {
         if (total > ctx->resid_cap) {
