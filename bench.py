@@ -196,7 +196,7 @@ def kernel_traffic(key):
 
 
 KERNEL_SOURCES = ("cg_persistent.cuh", "cg_persistent_body.cuh", "dslash_kernel.cuh", "link_codec.cuh",
-                  "hisq_internal.cuh", "solver_state.cuh", "ds_arith.cuh")
+                  "hisq_internal.cuh", "solver_state.cuh", "ds_arith.cuh", "dslash_mma.cuh")
 
 
 def kernel_source_hash():
