@@ -712,16 +712,6 @@ int hisq_links_create(hisq_links **out, const double *canon, int is_naik, int pr
         cudaMalloc(&h->scale, (size_t)2 * g.Vh * sizeof(float)) != cudaSuccess)
         rc = set_error(HISQ_ERR_NOMEM, "cannot allocate link scales");
     if (rc == HISQ_OK) dispatch_pack(prec, recon, g, U, hop, h->words, h->scale, h->W, st);
-    if (rc == HISQ_OK && prec >= HISQ_FP16 && recon == 18) {
-        // the tensor-core copy; without memory for it the other kernels serve the field
-        if (cudaMalloc(&h->frag, wbytes) == cudaSuccess) {
-            fragment_links_kernel<<<(int)((4L * g.Vh + 127) / 128), 128, 0, st>>>(g.Vh, h->words, h->frag,
-                                                                                prec == HISQ_BF16);
-        } else {
-            cudaGetLastError();
-            h->frag = nullptr;
-        }
-    }
     if (rc == HISQ_OK && prec != HISQ_FP64) {
         // the FP64 copy (plain FP64 solves with these links) and the double-single copy (the
         // residual recomputations of mixed-precision solves)
@@ -733,6 +723,17 @@ int hisq_links_create(hisq_links **out, const double *canon, int is_naik, int pr
             if (cudaMalloc(&h->words_ds, b64) != cudaSuccess)
                 rc = set_error(HISQ_ERR_NOMEM, "cannot allocate double-single link copy");
             else dispatch_pack(HISQ_DS, 18, g, U, hop, h->words_ds, nullptr, W64, st);
+        }
+    }
+    if (rc == HISQ_OK && prec >= HISQ_FP16 && recon == 18) {
+        // the tensor-core copy, after the copies that the handle cannot do without; without memory for it the
+        // other kernels serve the field
+        if (cudaMalloc(&h->frag, wbytes) == cudaSuccess) {
+            fragment_links_kernel<<<(int)((4L * g.Vh + 127) / 128), 128, 0, st>>>(g.Vh, h->words, h->frag,
+                                                                                prec == HISQ_BF16);
+        } else {
+            cudaGetLastError();
+            h->frag = nullptr;
         }
     }
     if (rc == HISQ_OK) {

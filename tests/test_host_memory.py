@@ -1,0 +1,79 @@
+"""The library's host code at the limits of device memory and with memory of another device, on a runtime
+without a GPU (fake_cudart.cpp): kernels do nothing there, so only statuses, allocations and copies count."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+FP16, BF16 = 2, 3
+DIMS = (8, 8, 8, 4)
+V = 8 * 8 * 8 * 4
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    from paper_1409_1510_gb300 import build
+    build.build()
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    out = str(tmp_path_factory.mktemp("fake") / "libhisq_fake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I", os.path.join(cuda, "include"),
+                    os.path.join(HERE, "fake_cudart.cpp")] + sorted(glob.glob(os.path.join(build.BUILD, "*.o")))
+                   + ["-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    lib.fake_used.restype = ctypes.c_size_t
+    lib.fake_refused.restype = ctypes.c_ulong
+    lib.fake_budget.argtypes = [ctypes.c_size_t]
+    lib.fake_foreign.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
+    lib.fake_copied.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.hisq_residual.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_double] + [ctypes.c_void_p] * 3 + [
+        ctypes.c_int, ctypes.c_void_p]
+    lib.cudaMalloc.argtypes = [ctypes.POINTER(ctypes.c_void_p), ctypes.c_size_t]
+    return lib
+
+
+@pytest.fixture
+def ctx(fake):
+    fake.fake_budget(ctypes.c_size_t(-1).value)
+    fake.fake_foreign(None, 0)
+    assert fake.hisq_init((ctypes.c_int * 4)(*DIMS), 0, None) == 0
+    yield fake
+    fake.fake_budget(ctypes.c_size_t(-1).value)
+    fake.fake_foreign(None, 0)
+    assert fake.hisq_finalize() == 0
+
+
+def _device(lib, nbytes):
+    p = ctypes.c_void_p()
+    assert lib.cudaMalloc(ctypes.byref(p), nbytes) == 0
+    return p.value
+
+
+def _links(lib, canon, naik, prec, recon=18):
+    h = ctypes.c_void_p()
+    return lib.hisq_links_create(ctypes.byref(h), ctypes.c_void_p(canon), naik, prec, recon), h
+
+
+@pytest.mark.parametrize("prec", [FP16, BF16])
+def test_links_fit_without_their_optional_copy(ctx, prec):
+    """Memory for the stored, FP64 and double-single records but not for the tensor-core copy too: the handle
+    is created, without that copy."""
+    canon = _device(ctx, 4 * V * 18 * 8)
+    before = ctx.fake_used()
+    rc, h = _links(ctx, canon, 0, prec)
+    assert rc == 0
+    whole = ctx.fake_used() - before
+    copy = V * 18 * 16  # as large as the 16-bit records: 8 links of 36 bytes per site
+    assert ctx.hisq_links_destroy(h) == 0 and ctx.fake_used() == before
+    for short in (1, copy // 2, copy):
+        ctx.fake_budget(before + whole - short)
+        rc, h = _links(ctx, canon, 0, prec)
+        assert rc == 0, short
+        assert ctx.fake_used() - before == whole - copy
+        assert ctx.hisq_links_destroy(h) == 0 and ctx.fake_used() == before
+    ctx.fake_budget(before + whole - copy - 1)
+    rc, h = _links(ctx, canon, 0, prec)
+    assert rc != 0 and ctx.fake_used() == before
