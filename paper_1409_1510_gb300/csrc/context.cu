@@ -31,13 +31,23 @@ int require_ctx(hisq_ctx **ctx) {
     return HISQ_OK;
 }
 
-bool is_device_ptr(const void *p) {
+static cudaPointerAttributes attributes_of(const void *p) {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        at.type = cudaMemoryTypeUnregistered;
     }
+    return at;
+}
+
+bool is_device_ptr(const void *p) {
+    const cudaPointerAttributes at = attributes_of(p);
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+bool on_device(const void *p, int device) {
+    const cudaPointerAttributes at = attributes_of(p);
+    return at.type == cudaMemoryTypeDevice && at.device == device;
 }
 
 int ensure_scratch(hisq_ctx *ctx, size_t partial_doubles, size_t tmp_bytes) {

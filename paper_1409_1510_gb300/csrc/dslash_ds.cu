@@ -189,10 +189,10 @@ extern "C" int hisq_residual(const hisq_links *fat, const hisq_links *naik, doub
     const size_t max_grid = (size_t)ctx->num_sms * 64;
     cudaStream_t st = ctx->stream;
     const bool ds = hp == LINKS_DS;
-    // The double-single kernels read b and x and write r in the canonical layout: caller's device buffers
-    // directly (16-byte aligned ones), others through a device copy.  Native FP64 goes through internal
-    // bundles and one staging buffer.
-    auto direct = [&](const void *p) { return ds && is_device_ptr(p) && (uintptr_t)p % 16 == 0; };
+    // The double-single kernels read b and x and write r in the canonical layout: caller's buffers directly
+    // (16-byte aligned ones in this device's own memory), others (host, managed, another device's) through a
+    // device copy.  Native FP64 goes through internal bundles and one staging buffer.
+    auto direct = [&](const void *p) { return ds && on_device(p, ctx->device) && (uintptr_t)p % 16 == 0; };
     const bool db = direct(rhs), dx = direct(x), dr = direct(r);
     const size_t pbytes = max_grid * nrhs * sizeof(double);
     const size_t staging = ds ? ((db ? 0 : canon) + (dx ? 0 : canon) + (dr ? 0 : canon)) : canon;

@@ -383,7 +383,8 @@ namespace hisq {
 hisq_ctx *current();
 int require_ctx(hisq_ctx **ctx);
 int ensure_scratch(hisq_ctx *ctx, size_t partial_doubles, size_t tmp_bytes);
-bool is_device_ptr(const void *p);
+bool is_device_ptr(const void *p);           // device memory of any device, or managed
+bool on_device(const void *p, int device);   // that device's own memory
 // Largest grid <= max_blocks that gives every block the same number of tiles (one fewer for
 // some when tiles is not a multiple), so no SM waits on a straggling extra tile.
 inline long balanced_grid(long tiles, long max_blocks) {

@@ -77,3 +77,35 @@ def test_links_fit_without_their_optional_copy(ctx, prec):
     ctx.fake_budget(before + whole - copy - 1)
     rc, h = _links(ctx, canon, 0, prec)
     assert rc != 0 and ctx.fake_used() == before
+
+
+@pytest.fixture
+def residual_buffers(ctx):
+    """(context, call, rhs, x, r): FP16 links and device buffers of hisq_residual for two right-hand sides."""
+    canon = _device(ctx, 4 * V * 18 * 8)
+    handles = [_links(ctx, canon, naik, FP16) for naik in (0, 1)]
+    assert [rc for rc, _ in handles] == [0, 0]
+    size = 2 * (V // 2) * 48
+    bufs = [_device(ctx, size + 4096) for _ in range(3)]
+
+    def call(rhs, x, r):
+        ctx.fake_clear()
+        assert ctx.hisq_residual(handles[0][1], handles[1][1], 0.1, rhs, x, r, 2, None) == 0
+        return [bool(ctx.fake_copied(rhs, 1)), bool(ctx.fake_copied(x, 1)), bool(ctx.fake_copied(r, 0))]
+
+    yield ctx, call, size, bufs
+    for p in bufs + [canon]:
+        ctx.cudaFree(ctypes.c_void_p(p))
+
+
+def test_residual_copies_buffers_of_another_device(residual_buffers):
+    """The kernels take buffers of the context's device as they are; those of another device, and host
+    memory, are copied."""
+    ctx, call, size, bufs = residual_buffers
+    assert call(*bufs) == [False, False, False]
+    for i, p in enumerate(bufs):
+        ctx.fake_foreign(p, size)
+        assert call(*bufs) == [j == i for j in range(3)]
+    ctx.fake_foreign(None, 0)
+    host = np.zeros((3, size), np.uint8)
+    assert call(*[host[i].ctypes.data for i in range(3)]) == [True, True, True]
