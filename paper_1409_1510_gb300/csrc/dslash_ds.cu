@@ -193,7 +193,12 @@ extern "C" int hisq_residual(const hisq_links *fat, const hisq_links *naik, doub
     // (16-byte aligned ones in this device's own memory), others (host, managed, another device's) through a
     // device copy.  Native FP64 goes through internal bundles and one staging buffer.
     auto direct = [&](const void *p) { return ds && on_device(p, ctx->device) && (uintptr_t)p % 16 == 0; };
-    const bool db = direct(rhs), dx = direct(x), dr = direct(r);
+    // the kernel that writes r still reads b and x: an r over part of either is written through the scratch
+    auto overlap = [&](const double *p, const double *q) {
+        const uintptr_t a = (uintptr_t)p, b = (uintptr_t)q;
+        return a < b + canon && b < a + canon;
+    };
+    const bool db = direct(rhs), dx = direct(x), dr = direct(r) && !overlap(r, rhs) && !overlap(r, x);
     const size_t pbytes = max_grid * nrhs * sizeof(double);
     const size_t staging = ds ? ((db ? 0 : canon) + (dx ? 0 : canon) + (dr ? 0 : canon)) : canon;
     const size_t total = staging + (ds ? 2 : 4) * vb + pbytes + 256;

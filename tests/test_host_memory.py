@@ -109,3 +109,21 @@ def test_residual_copies_buffers_of_another_device(residual_buffers):
     ctx.fake_foreign(None, 0)
     host = np.zeros((3, size), np.uint8)
     assert call(*[host[i].ctypes.data for i in range(3)]) == [True, True, True]
+
+
+def test_residual_stages_an_output_that_overlaps_an_input(residual_buffers):
+    """r over part of rhs or x: written through the scratch, so no input is overwritten while it is read."""
+    ctx, call, size, (b, x, r) = residual_buffers
+    one = size // 2
+    assert call(b, x, r) == [False, False, False]
+    for over in (b, x):
+        wide = _device(ctx, 3 * one)
+        # inputs in the first two thirds, r one right-hand side on; then the other way round; then the same
+        for at_in, at_r in ((wide, wide + one), (wide + one, wide), (wide, wide)):
+            args = [at_in if over == b else b, at_in if over == x else x, at_r]
+            assert call(*args)[2], (over == b, at_in - wide, at_r - wide)
+        assert call(wide if over == b else b, wide if over == x else x, r) == [False, False, False]
+        ctx.cudaFree(ctypes.c_void_p(wide))
+    wide = _device(ctx, 2 * size)
+    assert call(wide, x, wide + size) == [False, False, False]  # adjacent, not over one another
+    ctx.cudaFree(ctypes.c_void_p(wide))
