@@ -154,8 +154,9 @@ int hisq_aop(const hisq_links *fat, const hisq_links *naik, double mass, const v
  * exact products (Dekker 1971, by fused multiply-add) and error-free sums (Knuth's two-sum,
  * Ogita-Rump-Oishi cascaded summation) on the FP32 pipe, then b - m^2 x + D t in FP64; for FP64
  * handles native FP64.  rhs, x, r: host or device canonical double[nrhs][V/2][3][2] (r may alias
- * neither); res2: host or device double[nrhs] receiving |r_k|^2 (may be NULL).  Allocates its
- * scratch (cudaMalloc) for the call and synchronises the context's stream. */
+ * neither); res2: host or device double[nrhs] receiving |r_k|^2 (may be NULL).  Its scratch
+ * (cudaMalloc) is the context's and kept until hisq_finalize, up to 1 GiB; a call that needs more
+ * allocates and frees it.  Synchronises the context's stream. */
 int hisq_residual(const hisq_links *fat, const hisq_links *naik, double mass, const double *rhs,
                   const double *x, double *r, int nrhs, double *res2);
 
