@@ -136,47 +136,13 @@ __device__ __forceinline__ int tile_sites(int count, int spb) {
     return min(spb, (count + (int)gridDim.x - 1) / (int)gridDim.x);
 }
 
-// One thread's running dot product, in a form that stays off the FP64 pipe while it runs: an FP64 add or
-// conversion occupies that pipe for 16 cycles per warp and an SM has one, so two dots per site and
-// right-hand side cost as much as the loads they follow.  FP32 kernels form each site's dot in FP32; its
-// sum over the thread's sites and the lanes of a warp is a float pair, every addition a two-sum whose
-// error goes to the low part (48 significant bits), and becomes FP64 once per warp (64^3 x 16 FP16 solve:
-// A p phases 227 -> 212 ms; 32^3 x 8 single solve 4.60 -> 4.49 ms).  FP64 kernels add in FP64 throughout.
-template <typename T>
-struct DotSum;
-
-template <>
-struct DotSum<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double d) { v += d; }
-    __device__ __forceinline__ void add_lane(int off) { v += __shfl_xor_sync(0xffffffffu, v, off); }
-    __device__ __forceinline__ double value() const { return v; }
-};
-
-template <>
-struct DotSum<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void two_sum(float d) {
-        const float t = __fadd_rn(hi, d), z = __fsub_rn(t, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(d, z)));
-        hi = t;
-    }
-    __device__ __forceinline__ void add(float d) { two_sum(d); }
-    __device__ __forceinline__ void add_lane(int off) {
-        const float h = __shfl_xor_sync(0xffffffffu, hi, off), l = __shfl_xor_sync(0xffffffffu, lo, off);
-        lo = __fadd_rn(lo, l);
-        two_sum(h);
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Per-block column sums of the threads' dots into partials[blockIdx.x][col0 + *].  Thread
 // tid = site_row * t + gi holds dot[r] of column gi * cf + r * cs (by default gi * R + r; ndots columns).  With t a
 // power of two the lanes of one column meet in a shuffle tree and the warps' sums in one more
 // step; otherwise the dots go through red[rows][ndots] (red holds blockDim.x * R doubles).
 // With S lanes per thread position (tid = (site_row * t + gi) * S + part) the dots are in part 0.
-template <int R, int S = 1, typename T>
-__device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, DotSum<T> (&dot)[R], int t, int gi,
+template <int R, int S = 1>
+__device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, double (&dot)[R], int t, int gi,
                                              int ndots, int col0 = 0, int cf = R, int cs = 1) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int tS = t * S;
@@ -185,11 +151,11 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, Dot
     if ((t & (t - 1)) == 0 && tS <= 32) {
         for (int off = 16; off >= tS; off >>= 1)
 #pragma unroll
-            for (int r = 0; r < R; r++) dot[r].add_lane(off);
+            for (int r = 0; r < R; r++) dot[r] += __shfl_xor_sync(0xffffffffu, dot[r], off);
         if (lane < tS && own) {
 #pragma unroll
             for (int r = 0; r < R; r++)
-                if (gi * cf + r * cs < ndots) red[warp * ndots + gi * cf + r * cs] = dot[r].value();
+                if (gi * cf + r * cs < ndots) red[warp * ndots + gi * cf + r * cs] = dot[r];
         }
         __syncthreads();
         for (int j = warp; j < ndots; j += nwarps) {
@@ -206,7 +172,7 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, Dot
     if (row < rows && own) {
 #pragma unroll
         for (int r = 0; r < R; r++)
-            if (gi * cf + r * cs < ndots) red[row * ndots + gi * cf + r * cs] = dot[r].value();
+            if (gi * cf + r * cs < ndots) red[row * ndots + gi * cf + r * cs] = dot[r];
     }
     __syncthreads();
     for (int j = warp; j < ndots; j += nwarps) {
@@ -220,8 +186,8 @@ __device__ __forceinline__ void publish_dots(const PersArgs &a, double *red, Dot
 
 // The same for K sets of dots in one pass: dot[k][r] is column k step + gi R + r (n = t R,
 // step >= n); red holds K blockDim.x * R doubles.
-template <int R, int K, int S = 1, typename T>
-__device__ __forceinline__ void publish_dots_k(const PersArgs &a, double *red, DotSum<T> (&dot)[K][R], int t, int gi,
+template <int R, int K, int S = 1>
+__device__ __forceinline__ void publish_dots_k(const PersArgs &a, double *red, double (&dot)[K][R], int t, int gi,
                                                int n, int step) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int nd = K * n, tS = t * S;
@@ -234,13 +200,13 @@ __device__ __forceinline__ void publish_dots_k(const PersArgs &a, double *red, D
 #pragma unroll
             for (int k = 0; k < K; k++)
 #pragma unroll
-                for (int r = 0; r < R; r++) dot[k][r].add_lane(off);
+                for (int r = 0; r < R; r++) dot[k][r] += __shfl_xor_sync(0xffffffffu, dot[k][r], off);
         if (lane < tS && own) {
 #pragma unroll
             for (int k = 0; k < K; k++)
 #pragma unroll
                 for (int r = 0; r < R; r++)
-                    if (gi * R + r < n) red[warp * nd + k * n + gi * R + r] = dot[k][r].value();
+                    if (gi * R + r < n) red[warp * nd + k * n + gi * R + r] = dot[k][r];
         }
         __syncthreads();
         for (int j = warp; j < nd; j += nwarps) {
@@ -259,7 +225,7 @@ __device__ __forceinline__ void publish_dots_k(const PersArgs &a, double *red, D
         for (int k = 0; k < K; k++)
 #pragma unroll
             for (int r = 0; r < R; r++)
-                if (gi * R + r < n) red[row * nd + k * n + gi * R + r] = dot[k][r].value();
+                if (gi * R + r < n) red[row * nd + k * n + gi * R + r] = dot[k][r];
     }
     __syncthreads();
     for (int j = warp; j < nd; j += nwarps) {
@@ -344,7 +310,11 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
         act[r] = r0 + r < n && mask[r0 + r] != 0;
         any |= act[r];
     }
-    DotSum<real> dot[2][R];  // Re<ax, out>; with DOTS2 also |out|^2
+    double dot[2][R];  // Re<ax, out>; with DOTS2 also |out|^2
+#pragma unroll
+    for (int k = 0; k < 2; k++)
+#pragma unroll
+        for (int r = 0; r < R; r++) dot[k][r] = 0.0;
     const int ts = tile_sites(g.Vh, spb);
     if (S > 1 || (any && sl < ts)) {
         for (int tile = blockIdx.x; (long)tile * ts < g.Vh; tile += gridDim.x) {
@@ -399,12 +369,12 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
                         w[c] = {m2 * p[r][c].re - w[c].re, m2 * p[r][c].im - w[c].im};
                         d += p[r][c].re * w[c].re + p[r][c].im * w[c].im;
                     }
-                    dot[0][r].add(d);
+                    dot[0][r] += (double)d;
                     if constexpr (DOTS2) {
                         real f = 0;
 #pragma unroll
                         for (int c = 0; c < 3; c++) f += w[c].re * w[c].re + w[c].im * w[c].im;
-                        dot[1][r].add(f);
+                        dot[1][r] += (double)f;
                     }
                 }
                 store_adjacent<PP, R>(vout, s, r0, act, acc);
@@ -429,7 +399,7 @@ __device__ __forceinline__ void dslash_phase(const PersArgs &a, const LinkField 
                         d += wr * wr + wi * wi;
                         lo3[c] = {(typename Prec<Q>::real)wr, (typename Prec<Q>::real)wi};
                     }
-                    dot[0][r].add(d);
+                    dot[0][r] += d;
                     store_vec<Q>(vlo, s, r0 + r, lo3);
                 }
             }
@@ -460,7 +430,7 @@ __device__ __forceinline__ void mma_phase_n(const PersArgs &a, const void *in, v
         m2_hi = (float)m2v[min(L.r_hi, n - 1)];
     }
     const char *vin = mma_ptr(L, in), *vout = mma_ptr(L, out), *vax = mma_ptr(L, ax);
-    DotSum<float> sum;  // lane q of a quad: Re <p, w> of the two right-hand sides, |w|^2 of the two
+    double sum = 0.0;  // lane q of a quad: Re <p, w> of the two right-hand sides, |w|^2 of the two
     for (int u = blockIdx.x * nw + warp; u < R.count; u += gridDim.x * nw) {
         MmaRun run;
         if (!mma_run(g, R, u, parity, run)) continue;
@@ -468,14 +438,14 @@ __device__ __forceinline__ void mma_phase_n(const PersArgs &a, const void *in, v
             if constexpr (EPI == EPI_AOP) {
                 float d[4];
                 mma_aop<PP, N, true>(L, vax, s, m2_lo, m2_hi, w, d);
-                sum.add(mma_quad_sums(d, L.q));
+                sum += (double)mma_quad_sums(d, L.q);
             }
             mma_store(L, vout, s, w, L.has_lo, L.has_hi);
         });
     }
     if constexpr (EPI == EPI_AOP) {
         __syncthreads();  // red may still be read by the previous step
-        red[warp * 32 + lane] = sum.value();
+        red[warp * 32 + lane] = sum;
         __syncthreads();
         for (int col = warp; col < 32; col += nw) {  // one lane position per warp: a shuffle tree over the warps
             double s = lane < nw ? red[lane * 32 + col] : 0.0;
@@ -527,7 +497,9 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
         act[r] = gi + r * t < nlist;
         rr[r] = act[r] ? list[gi + r * t] : 0;
     }
-    DotSum<double> dot[DR];
+    double dot[DR];
+#pragma unroll
+    for (int r = 0; r < DR; r++) dot[r] = 0.0;
     const int ts = tile_sites(g.Vh, spb);
     if (S > 1 || sl < ts) {
         for (int tile = blockIdx.x; (long)tile * ts < g.Vh; tile += gridDim.x) {
@@ -573,7 +545,7 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
                         d += wr * wr + wi * wi;
                         lo3[c] = {(typename Prec<Q>::real)wr, (typename Prec<Q>::real)wi};
                     }
-                    dot[r].add(d);
+                    dot[r] += d;
                     store_vec<Q>(VecView<Q>{out_lo, n}, s, rr[r], lo3);
                 }
             }

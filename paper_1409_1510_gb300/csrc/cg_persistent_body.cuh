@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
 
     // ---- setup: x_hi = 0, x = 0, r = b, p = b and |b|^2 ----
     {
-        DotSum<double> acc[1];
+        double acc[1] = {0.0};
         if (row_ok) {
             for (int tile = blockIdx.x; (long)tile * ts < a.g.Vh; tile += gridDim.x) {
                 const int s = tile * ts + sl;
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
                 Cplx<rp> bp[3];
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
-                    acc[0].add(b[c].re * b[c].re + b[c].im * b[c].im);
+                    acc[0] += b[c].re * b[c].re + b[c].im * b[c].im;
                     bq[c] = {(rq)b[c].re, (rq)b[c].im};
                     bp[c] = {(rp)b[c].re, (rp)b[c].im};
                 }
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
         // x += alpha p; r -= alpha A p with |r|^2 (for the next iteration's step); p = r + beta p,
         // except where an FP64 recomputation is due (there x_hi += x, x = 0, and p waits for the
         // true residual)
-        DotSum<rq> rr_acc[1];
+        double rr_acc[1] = {0.0};
         if (st.active[r] && row_ok) {
             const rq al = (rq)st.alpha[r][0];
             const rp be = (rp)st.beta[r][0];
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
                 rq part = 0;
 #pragma unroll
                 for (int c = 0; c < 3; c++) part += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
-                rr_acc[0].add(part);
+                rr_acc[0] += (double)part;
                 if (upd) {
                     Cplx<double> xh[3];
                     const Cplx<rq> zq[3] = {{0, 0}, {0, 0}, {0, 0}};
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
         clock_mark(clk, PH_AOP);
         // x += alpha p; r -= alpha A p; |r|^2
         {
-            DotSum<rq> acc[1];
+            double acc[1] = {0.0};
             if (st.active[r] && row_ok) {
                 const rq al = (rq)st.alpha[r][0];
                 for (int tile = blockIdx.x; (long)tile * ts < a.g.Vh; tile += gridDim.x) {
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
                         rv[c].im -= al * (rq)ap[c].im;
                         part += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
                     }
-                    acc[0].add(part);
+                    acc[0] += (double)part;
                     store_vec<Q>(VQ(x), s, r, x);
                     store_vec<Q>(VQ(r), s, r, rv);
                 }

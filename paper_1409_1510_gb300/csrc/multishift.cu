@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(MS_PERS_THREADS, P == HISQ_FP64 ? 1 : 2) ms_pe
         }
         __syncthreads();
         // update pass: p_j, x_j for the live shifts; r -= alpha A p with |r|^2
-        DotSum<rq> acc[1];
+        double acc[1] = {0.0};
         if (s_ok) {
             const rq al = (rq)s_alpha;
             const int nl = s_nlive;
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(MS_PERS_THREADS, P == HISQ_FP64 ? 1 : 2) ms_pe
                     rv[c] = {rv[c].re - al * (rq)ap[c].re, rv[c].im - al * (rq)ap[c].im};
                     part += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
                 }
-                acc[0].add(part);
+                acc[0] += (double)part;
                 store_vec<Q>(vr, s, 0, rv);
             }
         }

@@ -290,3 +290,15 @@ def test_a_lane_per_link_group_on_small_lattices(prec, dims, n):
             x, stats, iters, res = _solve(g, rhs, 0.1, inner_prec=prec, bundle=n, single_reduction=single)
             true = g.oracle.true_residual(np.stack(rhs), x, 0.1)
             assert np.all(true <= TOL * SLACK), (single, true)
+
+
+@pytest.mark.parametrize("prec,n", [(1, 1), (1, 4), (2, 1), (2, 4), (3, 4)])
+@pytest.mark.parametrize("single_reduction", [0, 1])
+def test_dots_whose_running_sums_pass_the_float_range(prec, n, single_reduction):
+    """Right-hand sides of size 4e17: the |A p|^2 and |r|^2 of a site fit a float (1e38), their sums over a
+    thread's sites and a warp's lanes do not; they are FP64."""
+    dims, mass = (16, 16, 16, 8), 0.1
+    with gpu(dims, prec) as g:
+        rhs = [4e17 * hi.gaussian_rhs(g.lat, 900 + k) for k in range(n)]
+        x, stats, iters, res = _solve(g, rhs, mass, inner_prec=prec, bundle=n, single_reduction=single_reduction)
+        assert np.all(g.oracle.true_residual(np.stack(rhs), x, mass) <= TOL * SLACK)
