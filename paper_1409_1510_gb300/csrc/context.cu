@@ -399,7 +399,7 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
     const Geom &G = d.geom ? *d.geom : ctx->geom;
     LaunchShape sh = shape ? *shape : tuned_shape(ctx, fat, naik, d.n, copy);
     const bool mma = sh.S == 32 && mma_applies(fat, naik, copy, d);
-    if (sh.S == 32 && !mma) sh = default_shape(prec, d.n);  // buffers or links that kernel cannot take
+    if (sh.S == 32 && !mma) sh = simt_shape(ctx, prec, recon, d.n);  // what that kernel cannot take
     int R = sh.R;
     if (R != 1 && R != 2 && R != 4 && R != 8) R = 1;
     if (d.n % R != 0) R = 1;

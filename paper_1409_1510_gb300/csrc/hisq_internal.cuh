@@ -312,7 +312,7 @@ struct hisq_pc {
 namespace hisq {
 
 struct TuneKey {
-    int prec, recon, n, kind;
+    int prec, recon, n, kind;  // kind 0: the shape in use; 1: the fastest one of the SIMT kernels
     bool operator<(const TuneKey &o) const {
         if (prec != o.prec) return prec < o.prec;
         if (recon != o.recon) return recon < o.recon;
@@ -459,6 +459,7 @@ int launch_dslash(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, 
                   const DslashArgs &a, const LaunchShape *shape, cudaStream_t stream, int *grid_out = nullptr);
 LaunchShape default_shape(int prec, int n);
 LaunchShape tuned_shape(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, int n, int copy);
+LaunchShape simt_shape(hisq_ctx *ctx, int prec, int recon, int n);
 int choose_bundle(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *naik, int nrhs, int copy);  // tune.cu
 // the precision id a copy computes in (tuning keys, vector sizes)
 inline int copy_prec(const hisq_links *fat, int copy) {

@@ -95,7 +95,8 @@ static int run_tuner(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *nai
         if (rc != HISQ_OK) break;
     }
     // the tensor-core kernel, runs of 32, 16, 8 and 4 sites
-    if (copy == LINKS_INNER && mma_fields(fat, naik, n))
+    if (copy == LINKS_INNER && mma_fields(fat, naik, n) && rc == HISQ_OK) {
+        ctx->tuned[TuneKey{prec, recon, n, 1}] = *best;  // for the launches that kernel cannot take
         for (int run = 32; run >= 4 && rc == HISQ_OK; run /= 2) {
             LaunchShape sh{1, 32 * run, 32};
             float ms = 0;
@@ -105,6 +106,7 @@ static int run_tuner(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *nai
                 *best = sh;
             }
         }
+    }
     cudaStreamSynchronize(ctx->stream);
     cudaFree(in);
     cudaFree(out);
@@ -133,6 +135,14 @@ LaunchShape tuned_shape(hisq_ctx *ctx, const hisq_links *fat, const hisq_links *
     if (ms > 0.0f && ms < 1e29f) ctx->tuned_ms[key] = ms;
     ctx->tune_generation++;
     return best;
+}
+
+// The fastest shape of the other kernels where the tensor-core one was chosen or pinned (the default shape
+// when nothing was tuned).  Default against tuned here, decomposed BF16 Dslash at 64^3 x 16: 16 right-hand
+// sides 1.56 / 1.46 ms, 12: 1.46 / 1.23, 8: 0.839 / 0.809.
+LaunchShape simt_shape(hisq_ctx *ctx, int prec, int recon, int n) {
+    auto it = ctx->tuned.find(TuneKey{prec, recon, n, 1});
+    return it != ctx->tuned.end() ? it->second : default_shape(prec, n);
 }
 
 // Bundle size for nrhs right-hand sides: the candidate (1, 2, 4, 8, 12, 16 below

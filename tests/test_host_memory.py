@@ -1,5 +1,6 @@
-"""The library's host code at the limits of device memory and with memory of another device, on a runtime
-without a GPU (fake_cudart.cpp): kernels do nothing there, so only statuses, allocations and copies count."""
+"""The library's host code on a runtime without a GPU (fake_cudart.cpp): at the limits of device memory, with
+memory of another device, and which kernel a call is given.  Kernels do nothing there, so only statuses,
+allocations, copies and the names of the kernels count."""
 import ctypes
 import glob
 import os
@@ -28,6 +29,8 @@ def fake(tmp_path_factory):
     lib.fake_refused.restype = ctypes.c_ulong
     lib.fake_budget.argtypes = [ctypes.c_size_t]
     lib.fake_foreign.argtypes = [ctypes.c_void_p, ctypes.c_size_t]
+    lib.fake_time.argtypes = [ctypes.c_char_p, ctypes.c_float]
+    lib.fake_launched.argtypes = [ctypes.c_char_p]
     lib.fake_copied.argtypes = [ctypes.c_void_p, ctypes.c_int]
     lib.hisq_residual.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_double] + [ctypes.c_void_p] * 3 + [
         ctypes.c_int, ctypes.c_void_p]
@@ -43,6 +46,7 @@ def ctx(fake):
     yield fake
     fake.fake_budget(ctypes.c_size_t(-1).value)
     fake.fake_foreign(None, 0)
+    fake.fake_clear_times()
     assert fake.hisq_finalize() == 0
 
 
@@ -127,3 +131,30 @@ def test_residual_stages_an_output_that_overlaps_an_input(residual_buffers):
     wide = _device(ctx, 2 * size)
     assert call(wide, x, wide + size) == [False, False, False]  # adjacent, not over one another
     ctx.cudaFree(ctypes.c_void_p(wide))
+
+
+@pytest.mark.parametrize("R", [1, 2])
+def test_launches_the_tensor_cores_cannot_take_keep_the_tuned_shape(ctx, R):
+    """Where the tensor-core kernel is the fastest, the decomposed Dslash (which it cannot take) runs the
+    fastest of the other shapes, not the default one."""
+    lt = 8
+    assert ctx.hisq_finalize() == 0
+    assert ctx.hisq_init((ctypes.c_int * 4)(8, 8, 8, lt), 0, None) == 0
+    canon = _device(ctx, 8 * V * 18 * 8)
+    (rc0, fat), (rc1, naik) = (_links(ctx, canon, k, BF16) for k in (0, 1))
+    slabs = ctypes.c_void_p()
+    assert [rc0, rc1] == [0, 0]
+    assert ctx.hisq_slabs_create(ctypes.byref(slabs), ctypes.c_void_p(canon), ctypes.c_void_p(canon), BF16, 2) == 0
+    name = b"dslash_kernelILi%dELi18ELi%dELi0ELi2E" % (BF16, R)  # plain, two lanes per site
+    ctx.fake_time(name, 0.5)
+    ctx.fake_time(b"dslash_mma_kernel", 0.1)
+    n, shape = 8, [ctypes.c_int() for _ in range(3)]
+    assert ctx.hisq_autotune(fat, naik, n, *[ctypes.byref(v) for v in shape]) == 0
+    assert shape[2].value == 32
+    vec = _device(ctx, n * 8 ** 3 * lt // 2 * 48)
+    ctx.fake_clear()
+    assert ctx.hisq_slabs_dslash(slabs, ctypes.c_void_p(vec), ctypes.c_void_p(vec), n, 0, None) == 0
+    assert ctx.fake_launched(b"dslash_kernel") == ctx.fake_launched(name) > 0
+    assert ctx.hisq_slabs_destroy(slabs) == 0
+    for p in (canon, vec):
+        ctx.cudaFree(ctypes.c_void_p(p))
