@@ -876,6 +876,23 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     if (S.pc || S.naik->recon != 18) return HISQ_OK;
     Workspace *w = S.w;
     LaunchShape sh = tuned_shape(S.ctx, S.fat, S.naik, S.n, S.prec == HISQ_FP64 ? LINKS_FP64 : LINKS_INNER);
+    // a lattice so small that with one block per SM every site and right-hand side of a block's share gets
+    // four lanes, or as many as the precision allows (beyond that the lanes would take turns).  At 8^3 x 4 a
+    // block has seven sites: one lane each left 9200 cycles of FP64 multiply-adds in one chain of
+    // instructions with 25 lanes idle; plain FP64 CG there 3.20 ms, with four lanes 1.43, with 16 1.23
+    const long share = (S.ctx->geom.Vh + S.ctx->num_sms - 1) / S.ctx->num_sms;
+    int lanes = pers_most_lanes(S.prec);
+    if (share * S.n * lanes > PERS_DEFAULT_THREADS) lanes = 4;
+    const bool split = S.ctx->params.persistent_threads == 0 && share * S.n * lanes <= PERS_DEFAULT_THREADS;
+    // The tensor-core phases where the tuner found that kernel the fastest for this bundle and enough of a
+    // product's 16 rows are filled.  The separate kernel's time does not say it: between barriers the SIMT
+    // phases gain more.  us an iteration, SIMT / tensor-core phases, 64^3 x 16: FP16 8: 2371 / 3244,
+    // 9: 3224 / 3390, 10: 3056 / 3510, 11: 3956 / 3639, 12: 3583 / 3749, 13: 4700 / 3892, 14: 4206 / 3965,
+    // 16: 4627 / 4075 (odd ones run one per thread in the SIMT phases); BF16 8: 2676 / 2976, 10: 3318 / 3342,
+    // 12: 3944 / 3659, 14: 4552 / 4015, 16: 5147 / 4015.  32^3 x 8 draws the same line.
+    const bool mma = !split && sh.S == 32 && S.prec != HISQ_FP64 && S.n <= MMA_GROUP &&
+                     S.n > (S.prec == HISQ_BF16 || S.n % 2 ? 10 : 12) && mma_fields(S.fat, S.naik, S.n);
+    if (sh.S == 32 && !mma) sh = simt_shape(S.ctx, S.prec, S.naik->recon, S.n);
     int R = sh.R > 4 ? 4 : sh.R;
     if (S.prec == HISQ_FP64 && R > 2) R = 2;  // four FP64 right-hand sides per thread would spill
     // four FP32 right-hand sides per thread fit the separate Dslash kernel (up to 255 registers) but
@@ -885,17 +902,7 @@ static int solve_bundle_persistent(Solve &S, double tol, bool *done) {
     // right-hand sides.  FP16 keeps four (its records unpack into packed pairs): 3% faster there.
     if ((S.prec == HISQ_FP32 || S.prec == HISQ_BF16) && R > 2) R = 2;
     while (S.n % R) R /= 2;
-    // a lattice so small that with one block per SM every site and right-hand side of a block's share gets
-    // four lanes, or as many as the precision allows (beyond that the lanes would take turns).  At 8^3 x 4 a
-    // block has seven sites: one lane each left 9200 cycles of FP64 multiply-adds in one chain of
-    // instructions with 25 lanes idle; plain FP64 CG there 3.20 ms, with four lanes 1.43, with 16 1.23
-    const long share = (S.ctx->geom.Vh + S.ctx->num_sms - 1) / S.ctx->num_sms;
-    int lanes = pers_most_lanes(S.prec);
-    if (share * S.n * lanes > PERS_DEFAULT_THREADS) lanes = 4;
-    const bool split = S.ctx->params.persistent_threads == 0 && share * S.n * lanes <= PERS_DEFAULT_THREADS;
     if (split) R = 1;
-    // the tensor-core phases where the tuner found that kernel the fastest for this bundle
-    const bool mma = !split && sh.S == 32 && S.prec != HISQ_FP64 && S.n <= MMA_GROUP && mma_fields(S.fat, S.naik, S.n);
     if (mma) R = MMA_GROUP;
     // block size: the parameter if set (a multiple of 32 up to the kernel's bound), else 512
     int threads = std::min(pers_threads(R), PERS_DEFAULT_THREADS);

@@ -8,6 +8,8 @@ import hisq_inputs as hi
 import oracle
 
 PREC_TOL = {0: 1e-12, 1: 1e-5, 2: 5e-3, 3: 5e-3}   # per-Dslash norm-wise bound per precision
+# bundle sizes whose persistent solve takes the tensor-core phases where that kernel is the tuned one
+MMA_PHASES = {2: (11, 13, 14, 15, 16), 3: (12, 14, 16)}
 PREC_NAME = {0: "fp64", 1: "fp32", 2: "fp16", 3: "bf16"}
 
 

@@ -9,6 +9,8 @@ import subprocess
 import numpy as np
 import pytest
 
+from gpu_util import MMA_PHASES
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 FP16, BF16 = 2, 3
 DIMS = (8, 8, 8, 4)
@@ -158,3 +160,33 @@ def test_launches_the_tensor_cores_cannot_take_keep_the_tuned_shape(ctx, R):
     assert ctx.hisq_slabs_destroy(slabs) == 0
     for p in (canon, vec):
         ctx.cudaFree(ctypes.c_void_p(p))
+
+
+def _solve(lib, fat, naik, n, half_volume, **params):
+    """hisq_cg_solve of one bundle of n; the status is of no interest (no kernel runs)."""
+    from paper_1409_1510_gb300 import hisq
+    p = hisq.hisq_solver_params()
+    assert lib.hisq_default_solver_params(ctypes.byref(p)) == 0
+    p.bundle = n
+    for k, v in params.items():
+        setattr(p, k, v)
+    assert lib.hisq_set_solver_params(ctypes.byref(p)) == 0
+    vecs = [np.zeros((half_volume, 6)) for _ in range(2 * n)]
+    ptrs = [(ctypes.c_void_p * n)(*[v.ctypes.data for v in half]) for half in (vecs[:n], vecs[n:])]
+    lib.fake_clear()
+    lib.hisq_cg_solve(fat, naik, *ptrs, n, ctypes.c_double(0.1), ctypes.c_double(1e-10))
+
+
+@pytest.mark.parametrize("prec,phases", sorted(MMA_PHASES.items()))
+def test_persistent_tensor_core_phases_by_bundle_size(ctx, prec, phases):
+    """Where the separate Dslash is fastest on the tensor cores, the persistent solve takes its tensor-core
+    phases for the bundle sizes that they were measured faster at."""
+    canon = _device(ctx, 4 * V * 18 * 8)
+    (rc0, fat), (rc1, naik) = (_links(ctx, canon, k, prec) for k in (0, 1))
+    assert [rc0, rc1] == [0, 0]
+    ctx.fake_time(b"dslash_mma_kernel", 0.1)
+    for n in range(1, 17):
+        _solve(ctx, fat, naik, n, V // 2, inner_prec=prec, persistent_threads=512)
+        assert ctx.fake_launched(b"cg_persistent_kernel") == 1
+        assert ctx.fake_launched(b"cg_persistent_kernelILi%dELi16E" % prec) == (n in phases), n
+    ctx.cudaFree(ctypes.c_void_p(canon))
