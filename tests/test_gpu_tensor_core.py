@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import hisq_inputs as hi
-from gpu_util import PREC_TOL, gpu, rel_err
+from gpu_util import MMA_PHASES, PREC_TOL, gpu, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -52,6 +52,51 @@ def test_persistent_solve(prec, n, single_reduction):
         xs = [np.zeros_like(b) for b in rhs]
         g.hisq.hisq_cg_solve(g.fat, g.naik, rhs, xs, mass, tol)
         assert np.all(g.oracle.true_residual(np.stack(rhs), np.stack(xs), mass) <= tol)
+
+
+# The tensor-core phases of the persistent solve themselves: bundle sizes that take them (test_host_logic.py
+# checks that they do), with persistent_threads = 512, so that no small lattice is split over more lanes.
+# Rows of 4 and 8 sites (worked on 4 at a time; 16 right-hand sides with a layout known at compile time),
+# of 6 (2 at a time) and of 5 (one at a time); the last row group short at 10 x 6 x 6 x 6.
+@pytest.mark.parametrize("dims", [(8, 10, 8, 6), (16, 6, 4, 4), (12, 6, 6, 6), (10, 6, 6, 6)])
+@pytest.mark.parametrize("prec,n", [(p, n) for p in MMA_PHASES for n in MMA_PHASES[p]])
+@pytest.mark.parametrize("single_reduction", [0, 1])
+def test_persistent_phases(dims, prec, n, single_reduction):
+    mass, tol = 0.05, 1e-10
+    with gpu(dims, prec) as g:
+        g.hisq.hisq_set_launch_shape(prec, 18, n, 1, 128, LANES)
+        p = g.hisq.hisq_default_solver_params()
+        p.inner_prec, p.bundle, p.single_reduction, p.persistent_threads = prec, n, single_reduction, 512
+        g.hisq.hisq_set_solver_params(p)
+        rhs = list(_rhs(g.lat, n, 740))
+        rhs[1] = rhs[1] * 1e-3
+        rhs[2] = g.oracle.aop(g.oracle.aop(rhs[2], mass), mass)  # converges earlier than the others
+        rhs[n - 2] = np.zeros_like(rhs[0])                       # never active
+        xs = [np.full_like(b, 7.0) for b in rhs]
+        g.hisq.hisq_cg_solve(g.fat, g.naik, rhs, xs, mass, tol)
+        some = [k for k in range(n) if k != n - 2]
+        res = g.oracle.true_residual(np.stack([rhs[k] for k in some]), np.stack([xs[k] for k in some]), mass)
+        assert np.all(res <= tol) and not np.any(xs[n - 2])
+
+
+# The fused dots of this kernel and of a SIMT one on the same packed input.  Both sum exact products of the
+# stored values in FP32, 48 per component of D and a few scales, in different orders: for |D v| at most
+# sqrt(48) times its rounding-free terms' size, 48 roundings of 2^-24 are 3e-6 of a component, and the dot
+# averages over all of them; the stored intermediate differs where such a difference crosses a rounding
+# boundary of the storage (2^-24 48 against 2^-11 or 2^-9: one component in 170 or more, by one unit in the last
+# place, of random sign).  1e-5 of the dot holds both; the storage tolerance above is a thousand times wider.
+@pytest.mark.parametrize("dims", [(8, 10, 8, 4), (12, 4, 8, 6), (10, 6, 6, 6)])
+@pytest.mark.parametrize("prec,n", [(2, 9), (2, 16), (3, 10), (3, 16)])
+def test_fused_dots_agree_with_the_simt_kernel(dims, prec, n):
+    mass = 0.1
+    with gpu(dims, prec) as g:
+        vin, vout = g.pack(_rhs(g.lat, n, 760)), g.bundle(n)
+        dots = []
+        for shape in ((1, 128, LANES), (1, 128, 1)):
+            g.hisq.hisq_set_launch_shape(prec, 18, n, *shape)
+            dots.append(np.zeros(n))
+            g.hisq.hisq_aop(g.fat, g.naik, mass, vin, vout, n, dots[-1])
+        assert np.max(np.abs(dots[0] / dots[1] - 1.0)) <= 1e-5
 
 
 def test_shape_round_trip_and_validation():
