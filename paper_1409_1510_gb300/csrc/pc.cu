@@ -94,6 +94,7 @@ struct PcWork {
     int K = 0;
     float2 *h1[2] = {nullptr, nullptr}, *h2[2] = {nullptr, nullptr};  // 4 channels per parity
     float2 *k1[2] = {nullptr, nullptr}, *k2[2] = {nullptr, nullptr};  // the same for a second input (training)
+    bool k_tried = false;                 // the second set was asked for: there, or without memory for it
     float2 *g1[2] = {nullptr, nullptr}, *g2[2] = {nullptr, nullptr};
     float2 *y = nullptr, *G3 = nullptr;   // 1 channel, even
     float2 *u = nullptr, *d = nullptr;    // 1 channel, even: y - e and A (y - e)
@@ -166,9 +167,11 @@ static int ensure_work(hisq_ctx *ctx, hisq_pc *pc, int K) {
     return HISQ_OK;
 }
 
-// The second set of activations, for the workspace's K; false (and none kept) when memory is short.
+// The second set of activations, for the workspace's K; false (and none kept) when memory is short, which
+// is found out once per workspace: an allocation that fails costs as much as one that does not.
 static bool second_activations(hisq_ctx *ctx, PcWork &w) {
-    if (w.k1[0]) return true;
+    if (w.k_tried) return w.k1[0] != nullptr;
+    w.k_tried = true;
     const size_t f4 = (size_t)ctx->geom.Vh * 3 * w.K * 4 * sizeof(float2);
     float2 **bufs[] = {&w.k1[0], &w.k1[1], &w.k2[0], &w.k2[1]};
     for (float2 **b : bufs)

@@ -190,3 +190,35 @@ def test_persistent_tensor_core_phases_by_bundle_size(ctx, prec, phases):
         assert ctx.fake_launched(b"cg_persistent_kernel") == 1
         assert ctx.fake_launched(b"cg_persistent_kernelILi%dELi16E" % prec) == (n in phases), n
     ctx.cudaFree(ctypes.c_void_p(canon))
+
+
+def test_training_asks_for_its_optional_activations_once(ctx):
+    """Memory for the network's workspace but not for the second set of activations: the calls work without
+    it and do not try its allocations again, until the workspace itself is made anew."""
+    FP32 = 1
+    canon = _device(ctx, 4 * V * 18 * 8)
+    (rc0, fat), (rc1, naik) = (_links(ctx, canon, k, FP32) for k in (0, 1))
+    pc, loss, grad = ctypes.c_void_p(), ctypes.c_double(), np.zeros(408 * 2)
+    assert [rc0, rc1, ctx.hisq_pc_create(ctypes.byref(pc), None)] == [0, 0, 0]
+    vec = _device(ctx, 3 * V // 2 * 24)
+
+    def call(K):
+        before = ctx.fake_refused()
+        assert ctx.hisq_pc_loss_grad(pc, fat, naik, ctypes.c_double(0.1), ctypes.c_void_p(vec), ctypes.c_void_p(vec),
+                                     K, ctypes.byref(loss), ctypes.c_void_p(grad.ctypes.data)) == 0
+        return ctx.fake_refused() - before
+
+    one = V // 2 * 3 * 4 * 8  # a set of activations is four of these per sample
+    for K in (1, 2):
+        ctx.fake_budget(ctypes.c_size_t(-1).value)
+        assert call(K) == 0  # the whole workspace for K fits
+        whole = ctx.fake_used()
+        assert ctx.hisq_pc_destroy(pc) == 0 and ctx.hisq_pc_create(ctypes.byref(pc), None) == 0
+        ctx.fake_budget(whole - 4 * K * one + 3 * K * one)
+        assert [call(K) for _ in range(3)] == [1, 0, 0]
+        assert ctx.fake_used() == whole - 4 * K * one
+    ctx.fake_budget(ctypes.c_size_t(-1).value)
+    assert call(3) == 0 and ctx.fake_used() > whole  # a larger workspace asks again
+    assert ctx.hisq_pc_destroy(pc) == 0
+    for p in (canon, vec):
+        ctx.cudaFree(ctypes.c_void_p(p))
