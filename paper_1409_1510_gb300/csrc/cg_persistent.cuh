@@ -477,13 +477,13 @@ __device__ __forceinline__ void mma_phase(const PersArgs &a, const void *in, voi
 // right-hand sides list[gi + r t] (nlist listed in all, t = ceil(nlist / DR) threads per site).  Kernels
 // with more than one right-hand side per thread take DR = 2: two share each link load and give a thread
 // twice the independent chains.
-// PF: prefetch the next link's operands (it made the persistent kernels spill, so they pass
-// false; the separate kernels of dslash_ds.cu prefetch).
+// The next link's operands are not requested ahead (that made these kernels spill; the separate kernels of
+// dslash_ds.cu do it).
 // EPI_PLAIN: out = D in (ds bundles).  EPI_RESID: r = b - m^2 x + D in with x, b FP64
 // and an FP64 epilogue, written to out_lo in the iterated precision Q, with |r|^2 per block
 // published as column i of the list.
 // S > 1: S lanes per (site, right-hand side) on small lattices (see dslash_phase).
-template <int EPI, int Q, int DR, bool PF, int S = 1>
+template <int EPI, int Q, int DR, int S = 1>
 __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void *out, int parity, const void *xvec,
                                          const void *bvec, void *out_lo, double *red, const double *m2v,
                                          const int *list, int nlist) {
@@ -509,12 +509,12 @@ __device__ __forceinline__ void ds_phase(const PersArgs &a, const void *in, void
             const int s = visit_site(g, valid ? q : 0);
             dscplx acc[DR][3];
             if constexpr (S == 1) {
-                ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
+                ds_site_stencil<DR, true>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
                                               rr, act, acc);
             } else {
                 constexpr int PAIRS = 8 / S;  // (kind, direction) pairs per lane
                 static_assert(S == 4 || S == 8, "a lane takes both hops of its directions");
-                ds_site_stencil<DR, true, PF>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
+                ds_site_stencil<DR, true>(g, a.fat64, a.naik64, parity, reinterpret_cast<const float4 *>(in), n, s,
                                               rr, act, acc, PAIRS * part, valid ? PAIRS * (part + 1) : PAIRS * part);
 #pragma unroll
                 for (int off = 1; off < S; off <<= 1)  // every lane of the warp takes part
@@ -563,7 +563,7 @@ template <int EPI, int Q, int DR>
 __device__ __noinline__ void ds_phase_called(const PersArgs &a, const void *in, void *out, int parity,
                                              const void *xvec, const void *bvec, void *out_lo, double *red,
                                              const double *m2v, const int *list, int nlist) {
-    ds_phase<EPI, Q, DR, false>(a, in, out, parity, xvec, bvec, out_lo, red, m2v, list, nlist);
+    ds_phase<EPI, Q, DR>(a, in, out, parity, xvec, bvec, out_lo, red, m2v, list, nlist);
 }
 
 // x_hi of one site and right-hand side, written in double-single form for the recomputation

@@ -40,12 +40,17 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
 #define DS_PHASE(EPI, in, out, parity, x, b, lo)                                                             \
     do {                                                                                                     \
         if constexpr (R == 1)                                                                                \
-            ds_phase<EPI, Q, 1, false, S>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);     \
+            ds_phase<EPI, Q, 1, S>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);            \
         else if (upd_n == 1)                                                                                 \
             ds_phase_called<EPI, Q, 1>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);        \
         else                                                                                                 \
             ds_phase_called<EPI, Q, 2>(a, in, out, parity, x, b, lo, red, st.mass2, upd_list, upd_n);        \
     } while (0)
+    // the same halves in FP64 kernels
+#define FP64_PHASE(EPI, f, out, parity, b, lo, list, nlist)                                                           \
+    dslash_phase<HISQ_FP64, 1, EPI, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(                 \
+        a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(f)}, out, parity, st.update,                               \
+        PlainIn<HISQ_FP64, true>{V64(xhi)}, b, lo, red, st.mass2, list, nlist)
 
     // ---- setup: x_hi = 0, x = 0, r = b, p = b and |b|^2 ----
     {
@@ -162,13 +167,9 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
             }
             __syncthreads();
             if constexpr (P == HISQ_FP64) {
-                dslash_phase<HISQ_FP64, 1, EPI_PLAIN, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.t64,
-                                                         1, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, nullptr,
-                                                         nullptr, red, st.mass2, upd_list, upd_n);
+                FP64_PHASE(EPI_PLAIN, xhi, a.t64, 1, nullptr, nullptr, upd_list, upd_n);
                 if (!(ok = grid_sync(a))) break;
-                dslash_phase<HISQ_FP64, 1, EPI_RESID, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(t64)},
-                                                         nullptr, 0, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.b,
-                                                         a.r, red, st.mass2, upd_list, upd_n);
+                FP64_PHASE(EPI_RESID, t64, nullptr, 0, a.b, a.r, upd_list, upd_n);
             } else {
                 DS_PHASE(EPI_PLAIN, a.xds, a.t64, 1, nullptr, nullptr, nullptr);
                 if (!(ok = grid_sync(a))) break;
@@ -274,13 +275,9 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
             }
             if (!(ok = grid_sync(a))) break;
             if constexpr (P == HISQ_FP64) {
-                dslash_phase<HISQ_FP64, 1, EPI_PLAIN, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.t64,
-                                                         1, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, nullptr,
-                                                         nullptr, red, st.mass2);
+                FP64_PHASE(EPI_PLAIN, xhi, a.t64, 1, nullptr, nullptr, nullptr, 0);
                 if (!(ok = grid_sync(a))) break;
-                dslash_phase<HISQ_FP64, 1, EPI_RESID, Q, PlainIn<HISQ_FP64, true>, PlainIn<HISQ_FP64, true>, false, S>(a, a.fat64, a.naik64, PlainIn<HISQ_FP64, true>{V64(t64)},
-                                                         nullptr, 0, st.update, PlainIn<HISQ_FP64, true>{V64(xhi)}, a.b,
-                                                         a.r, red, st.mass2);
+                FP64_PHASE(EPI_RESID, t64, nullptr, 0, a.b, a.r, nullptr, 0);
                 if (!(ok = grid_sync(a))) break;
                 sum_partials(a, red, n, dots);
             } else {
@@ -326,6 +323,7 @@ __global__ void __launch_bounds__(pers_threads(R, S), 1) cg_persistent_kernel(co
     }
 #undef DSLASH
 #undef DS_PHASE
+#undef FP64_PHASE
 #undef V64
 #undef VQ
 #undef VP

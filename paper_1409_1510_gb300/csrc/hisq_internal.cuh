@@ -82,7 +82,7 @@ __host__ __device__ __forceinline__ int visit_site(const Geom &g, int q) {
     return within + P * (z + g.L[2] * t);
 }
 
-// even-odd index of the neighbour `step` hops (|step| <= 3 < L) away in direction mu// even-odd index of the neighbour `step` hops (|step| <= 3 < L) away in direction mu
+// even-odd index of the neighbour `step` hops (|step| <= 3 < L) away in direction mu
 __host__ __device__ __forceinline__ int neighbour(const Geom &g, const SiteCoord &sc, int s, int mu, int step) {
     int c = sc.c[mu] + step;
     int L = g.L[mu];
