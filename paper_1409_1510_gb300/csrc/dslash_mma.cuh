@@ -15,11 +15,17 @@
 //         lane's rows are right-hand sides 2 g and 2 g + 1, one 8-byte load.  Lanes q = 3 share
 //         component 0 with lanes q = 0, each against half of its link entries (zeros in one of them
 //         would turn an infinity into NaN).
-// Products of 16-bit values are exact and sums are FP32, as in the SIMT kernels, which spend two
-// thirds of their FMA-pipe cycles on the 36 products of every link and right-hand side and a fifth on
-// conversions.  Here what is left is loads, addresses and scales, and the latency of the loads (half of
-// the warps' time; it is that of L1 and L2: lattices within L2 take as long per site, and requests into L2
-// ahead of use only slowed it down).
+// Products of 16-bit values are exact and accumulators FP32 wide, but the tensor core adds with its own
+// rounding, towards zero: against 64-bit sums of the same stored values (16^3 x 8 and 28 x 20 x 12 x 10, 2 to
+// 16 right-hand sides) an FP16 output's largest component is off by 7.6e-8 rms, 3.4e-8 of it common to all;
+// SIMT kernels by 2.1e-7 rms and nothing in common.  A dot product over the lattice averages the rms away and
+// keeps the common part: 3.4e-8 (FP16) and 5.5e-8 (BF16) of it, SIMT 1e-9.  Rounding the links and
+// vectors to 16 bits puts far more on the same dots (BF16 at 28 x 20 x 36 x 10: 9.6e-6).
+//
+// The SIMT kernels spend two thirds of their FMA-pipe cycles on the 36 products of every link and right-hand
+// side and a fifth on conversions.  Here what is left is loads, addresses and scales, and the latency of the
+// loads (half of the warps' time; it is that of L1 and L2: lattices within L2 take as long per site, and
+// requests into L2 ahead of use only slowed it down).
 //
 // A warp visits a run of consecutive sites of one x-row, U at a time: the hops in y, z and t are then
 // the same index offsets for the whole run, U sites share the addresses of those neighbours, and their
@@ -395,12 +401,13 @@ __device__ __forceinline__ void mma_run_sites(const Geom &g, const MmaField &fat
     }
 }
 
-// Separate kernel: EPI_PLAIN or EPI_AOP of a whole parity, n <= MMA_MAX_N right-hand sides in a.t groups
-// (warps of a block alternate over the groups); a.spb = sites per run, a multiple of U.
-// Resident blocks per SM that the register budget is set for (measured with U = 4 at 64^3 x 16): FP16 2
-// (16 right-hand sides 990 us; 3: 1033, 4: 1205), BF16 3 with N = 16 (647; 2: 699) and N = 8, else 2.
+// Resident blocks per SM that the register budget of the separate kernel is set for (measured with U = 4 at
+// 64^3 x 16): FP16 2 (16 right-hand sides 990 us; 3: 1033, 4: 1205), BF16 3 with N = 16 (647; 2: 699) and
+// N = 8, else 2.
 constexpr int mma_blocks(int P, int N) { return P == HISQ_BF16 && N ? 3 : 2; }
 
+// Separate kernel: EPI_PLAIN or EPI_AOP of a whole parity, n <= MMA_MAX_N right-hand sides in a.t groups
+// (warps of a block alternate over the groups); a.spb = sites per run, a multiple of U.
 template <int P, int EPI, int N, int U>
 __global__ void __launch_bounds__(MMA_THREADS, mma_blocks(P, N)) dslash_mma_kernel(KArgs a, MmaField fat, MmaField naik) {
     extern __shared__ double red[];

@@ -234,6 +234,9 @@ __global__ void __launch_bounds__(256, pc_layer_blocks(A, B, NR)) pc_layer_kerne
 // and link kinds 14.6 -> 13.9 ms (between the two the forward activations were kept instead of
 // recomputed); with the blocks' sums added in groups (grad_finish) and three blocks per SM for the layers
 // of four weights 13.9 -> 12.95 ms.
+// Lanes add up to eight (site, sample) pairs in FP32 before the warp's tree and the FP64 sum, one before:
+// the gradient's error against 64 bits on eight lattices of 6400 to 110592 sites with 2 to 16 samples is
+// 3.6e-8 to 8.4e-8 either way (geometric mean of the 16 ratios 0.997).
 struct PcGradArgs {
     PcLayerArgs L;       // in_same, in_opp: the layer input h; spb: sites per tile; out unused
     const float2 *G;     // gradient w.r.t. the layer output at the output parity

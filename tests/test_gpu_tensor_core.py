@@ -80,11 +80,12 @@ def test_persistent_phases(dims, prec, n, single_reduction):
 
 
 # The fused dots of this kernel and of a SIMT one on the same packed input.  Both sum exact products of the
-# stored values in FP32, 48 per component of D and a few scales, in different orders: for |D v| at most
-# sqrt(48) times its rounding-free terms' size, 48 roundings of 2^-24 are 3e-6 of a component, and the dot
-# averages over all of them; the stored intermediate differs where such a difference crosses a rounding
-# boundary of the storage (2^-24 48 against 2^-11 or 2^-9: one component in 170 or more, by one unit in the last
-# place, of random sign).  1e-5 of the dot holds both; the storage tolerance above is a thousand times wider.
+# stored values in FP32 accumulators, 48 per component of D and a few scales, the tensor core with its own
+# rounding (towards zero, one unit of 2^-23 for each addition at the most): a component is off by at most
+# 48 2^-23 = 6e-6 of its terms' size, a dot by the part of that which all components have in common.  The
+# stored intermediate differs where such a difference crosses a rounding boundary of the storage (one component
+# in thousands, by one unit in the last place, of random sign).  1e-5 of the dot holds both; the storage
+# tolerance above is a thousand times wider.
 @pytest.mark.parametrize("dims", [(8, 10, 8, 4), (12, 4, 8, 6), (10, 6, 6, 6)])
 @pytest.mark.parametrize("prec,n", [(2, 9), (2, 16), (3, 10), (3, 16)])
 def test_fused_dots_agree_with_the_simt_kernel(dims, prec, n):
