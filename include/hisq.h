@@ -104,8 +104,9 @@ const char *hisq_last_error(void);
  * or, for Naik links only, 13 (two rows of W plus c, where N = c W, W in SU(3)) or 9 (eight
  * SU(3) parameters plus c); 13 and 9 are exact only for links of that form (Sec. 2: Naik links
  * can be rebuilt from 9 or 13/14 reals; fat links cannot).  16-bit 18-real links carry one
- * float scale per site and are kept a second time in the order of the tensor-core kernel (if memory
- * allows).  When prec != HISQ_FP64 the handle also keeps an FP64 copy, used by the
+ * float scale per site and are kept a second time in the order of the tensor-core kernel (288 bytes
+ * per site of the lattice; where memory does not allow it, the other kernels serve the handle).
+ * When prec != HISQ_FP64 the handle also keeps an FP64 copy, used by the
  * solvers' FP64 residual recomputation.  The input is not retained. */
 int hisq_links_create(hisq_links **h, const double *canon, int is_naik, int prec, int recon);
 int hisq_links_destroy(hisq_links *h);
@@ -420,7 +421,9 @@ int hisq_pc_set_form(hisq_pc *pc, int form);
  * with P = M^dag M (HISQ_PC_NORMAL) or P = M (HISQ_PC_HERMITIAN_PART), i.e. the error of the
  * preconditioner's correction measured in the residual norm, and its gradient
  * dL/dRe W + i dL/dIm W (host or device double[HISQ_PC_WEIGHTS][2]); r, e: device FP32 internal
- * bundles of K (1..HISQ_MAX_BUNDLE) vectors each. */
+ * bundles of K (1..HISQ_MAX_BUNDLE) vectors each.  The handle keeps a workspace for
+ * the largest K so far until it is destroyed: 468 bytes per sample and site of the lattice, and for
+ * M^dag M, where memory allows, 192 more. */
 int hisq_pc_loss_grad(const hisq_pc *pc, const hisq_links *fat, const hisq_links *naik, double mass,
                       const void *r, const void *e, int K, double *loss, double *grad);
 
