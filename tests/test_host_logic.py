@@ -2,7 +2,6 @@
 memory of another device, and which kernel a call is given.  Kernels do nothing there, so only statuses,
 allocations, copies and the names of the kernels count."""
 import ctypes
-import glob
 import os
 import subprocess
 
@@ -21,11 +20,11 @@ V = 8 * 8 * 8 * 4
 def fake(tmp_path_factory):
     from paper_1409_1510_gb300 import build
     build.build()
+    objects = [os.path.join(build.BUILD, os.path.basename(f)[:-3] + ".o") for f in build.sources()]
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     out = str(tmp_path_factory.mktemp("fake") / "libhisq_fake.so")
     subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I", os.path.join(cuda, "include"),
-                    os.path.join(HERE, "fake_cudart.cpp")] + sorted(glob.glob(os.path.join(build.BUILD, "*.o")))
-                   + ["-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", out], check=True)
+                    os.path.join(HERE, "fake_cudart.cpp")] + objects + ["-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", out], check=True)
     lib = ctypes.CDLL(out)
     lib.fake_used.restype = ctypes.c_size_t
     lib.fake_refused.restype = ctypes.c_ulong
