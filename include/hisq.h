@@ -371,7 +371,9 @@ int hisq_autotune(const hisq_links *fat, const hisq_links *naik, int nrhs, int *
  * memory by the bulk-copy engine (18-real Naik, FP32/FP16/BF16, rhs_per_thread <= 2; tiles of
  * block_threads / (4 nrhs / rhs_per_thread) sites, block_threads up to 512), or 32: one warp per site
  * on the tensor cores (18-real Naik, FP16 or BF16, 2..32 right-hand sides, an even number for BF16,
- * rhs_per_thread 1; block_threads = 32 times the 1..32 sites of a row that a warp visits in one go).
+ * rhs_per_thread 1; block_threads = 32 times the 1..32 sites of a row that a warp visits in one go;
+ * the persistent kernel of hisq_cg_solve follows that shape for bundles of 11 and 13..16 (FP16) or 12, 14
+ * and 16 (BF16), where its tensor-core phases are the faster ones).
  * Overrides the autotuner's choice for that key. */
 int hisq_set_launch_shape(int prec, int recon, int nrhs, int rhs_per_thread, int block_threads,
                           int lanes_per_site);
